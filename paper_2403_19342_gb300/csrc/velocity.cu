@@ -40,20 +40,20 @@ __global__ void k_velocity(const double* __restrict__ p, const double* __restric
                            int nx, int ny, int nz, double hx, double hy, double hz, int bx, int by, int bz,
                            const int* __restrict__ lex_of_hid, const int* __restrict__ nbr, int gx, int gy,
                            double* __restrict__ v, RedSlot red, double* out) {
-  const int64_t n = (int64_t)nx * ny * nz;
-  const int nb = bx * by * bz;
+  const unsigned n = (unsigned)nx * ny * nz;             // at most 2^31 - 1
+  const unsigned nb = (unsigned)(bx * by * bz);
   const double mean = out[0];
+  const double h[3] = {hx, hy, hz}, rh[3] = {1.0 / hx, 1.0 / hy, 1.0 / hz};
+  const int64_t st[3] = {1, nx, (int64_t)nx * ny};
+  const int bd[3] = {bx, by, bz}, lst[3] = {1, bx, bx * by}, nn[3] = {nx, ny, nz};
   double acc[2] = {0.0, 0.0};
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = i / nb;
-    const int q = (int)(i % nb);
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const unsigned e = i / nb;
+    const int q = (int)(i - e * nb);
     const int lex = lex_of_hid[e];
-    const int ex = lex % gx, ey = (lex / gx) % gy, ez = lex / (gx * gy);
+    const int ey0 = lex / gx, ex = lex - ey0 * gx, ez = ey0 / gy, ey = ey0 - ez * gy;
     const int lc[3] = {q % bx, (q / bx) % by, q / (bx * by)};
     const int gc[3] = {ex * bx + lc[0], ey * by + lc[1], ez * bz + lc[2]};
-    const int nn[3] = {nx, ny, nz}, bd[3] = {bx, by, bz}, lst[3] = {1, bx, bx * by};
-    const double h[3] = {hx, hy, hz};
-    const int64_t st[3] = {1, nx, (int64_t)nx * ny};
     const int64_t c = gc[0] + (int64_t)nx * (gc[1] + (int64_t)ny * gc[2]);
     const double pc = p[c];
     double div = 0.0;
@@ -68,14 +68,19 @@ __global__ void k_velocity(const double* __restrict__ p, const double* __restric
       if (gc[d] > 0) {
         int64_t im;
         if (lc[d] > 0) {
-          im = i - lst[d];
+          im = (int64_t)i - lst[d];
         } else {
-          const int ne = nbr[e * 6 + 2 * d];
+          const int ne = nbr[e * 6u + 2 * d];
           im = (int64_t)ne * nb + q + (int64_t)(bd[d] - 1) * lst[d];
         }
         vm = -T[(int64_t)d * n + im] * h[d] * (pc - p[c - st[d]]);
       }
-      div += (vp - vm) / h[d];
+      // (vp - vm) / h: the product with 1 / h and Markstein's correction (correctly
+      // rounded, in three FP64 instructions; the kernel is bound by the FP64 pipe)
+      const double dv = vp - vm;
+      double t = dv * rh[d];
+      if ((((uint64_t)__double_as_longlong(t) >> 52) & 0x7ff) != 0x7ff) t = fma(fma(-h[d], t, dv), rh[d], t);
+      div += t;
     }
     // the cell's net source: f - mean (the singular system), or f - W p with a cell
     // term (wells: the flow leaves through the well, not through a face)
