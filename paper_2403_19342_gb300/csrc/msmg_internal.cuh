@@ -182,8 +182,8 @@ struct SolveBuffers {
 }  // namespace msmg
 
 namespace msmg {
-// pivots per pass of the blocked Gauss-Jordan inversion of the coarsest matrix
-constexpr int kGjBlock = 4;
+// pivots per block of the coarsest matrix's inversion
+constexpr int kGjBlock = 32;
 }
 
 struct msmg_ctx {

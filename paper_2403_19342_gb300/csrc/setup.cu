@@ -13,7 +13,7 @@
 //    the Galerkin blocks of A_{l+1}; the parent's face terms; and the inverse
 //    of the parent's diagonal block (the block-Jacobi smoother of level l).
 //  * Coarsest level: A_L + sigma z z^T / |z|^2 (z spans null(A_L)) is inverted
-//    by Gauss-Jordan elimination and projected, giving the Moore-Penrose
+//    by symmetric block sweeps and projected, giving the Moore-Penrose
 //    inverse A_L^dagger used by Algorithm 1's coarsest correction.
 #include "msmg_internal.cuh"
 #include "reduce.cuh"
@@ -289,7 +289,13 @@ __device__ bool ic0_factor(const double* A, double* Lf, int nP, int L, int rx, i
 // keeps its candidates with eigenvalue below B, at least one; its other rows of
 // Psi are zero and its count goes to nx.cnt.  With given (imported) bases the
 // count is the number of leading nonzero rows of Psi.
-__global__ void k_coarse_setup(CoarseLevel lv, CoarseLevel nx, double* stats, int given, int ic0, double B) {
+//
+// The Ln smallest eigenpairs come from a tridiagonalisation (tridiag_eig: 4/3 nP^3 FP64
+// operations, where cyclic Jacobi spends 80 nP^3 or more); Jacobi on the whole matrix
+// where that does not reach its accuracy or its work space does not fit (tri_work: its
+// doubles, 0 for none).  512 parents of 48 unknowns 14.4 -> 2.7 ms, 935 of 60 34.8 -> 5.3 ms.
+__global__ void k_coarse_setup(CoarseLevel lv, CoarseLevel nx, double* stats, int given, int ic0, double B,
+                               int tri_work) {
   extern __shared__ double sm[];
   const int nP = lv.nP, L = lv.L, L2 = L * L, Ln = lv.Lnext, Ln2 = Ln * Ln;
   double* A = sm;                 // parent's diagonal block of A_l
@@ -301,6 +307,7 @@ __global__ void k_coarse_setup(CoarseLevel lv, CoarseLevel nx, double* stats, in
   int* order = pr + nP + 2;
   int* ridx = order + nP + 2;     // [nP] kept coordinates of the parent, in order
   int* cidx = ridx + nP;          // [nP] compact index of each coordinate (-1: unused slot)
+  double* tri = sm + 3 * nP * nP + (2 * nP + 4 + 72) + (4 * nP + 4 + 1) / 2 + 8;   // beyond jac_smem
   __shared__ int s_nr, s_cnt;
   const int64_t P = blockIdx.x;
   const int rx = lv.rx, ry = lv.ry;
@@ -353,29 +360,40 @@ __global__ void k_coarse_setup(CoarseLevel lv, CoarseLevel nx, double* stats, in
   const int nR = s_nr;
   if (!given) {
     // the local problem on the kept coordinates (all of them under Strategy 1)
+    const int nc = Ln < nR ? Ln : nR;
     for (int idx = threadIdx.x; idx < nR * nR; idx += blockDim.x)
       V[idx] = N[ridx[idx / nR] * nP + ridx[idx % nR]];
     __syncthreads();
-    jacobi_eig(V, N, nR, cs, pr, red, 40, 1e-15);
-    sort_diag(V, nR, order);
-    const int nc = Ln < nR ? Ln : nR;
+    const bool direct = tri_work > 0 && tridiag_eig(V, nR, nc, tri);
+    double* const lamv = tri;                            // direct: eigenvalues and vectors as tridiag_eig leaves them
+    const double* const Z = tri + tri_vectors(nR);
+    if (!direct) {
+      __syncthreads();
+      for (int idx = threadIdx.x; idx < nR * nR; idx += blockDim.x)
+        V[idx] = N[ridx[idx / nR] * nP + ridx[idx % nR]];
+      __syncthreads();
+      jacobi_eig(V, N, nR, cs, pr, red, 40, 1e-15);
+      sort_diag(V, nR, order);
+    }
+    auto lam_of = [&](int j) { return direct ? lamv[j] : V[order[j] * nR + order[j]]; };
     if (threadIdx.x == 0) {
       int cn = nc;
       if (B > 0.0) {
         cn = 0;
-        for (int j = 0; j < nc; ++j) cn += V[order[j] * nR + order[j]] < B ? 1 : 0;
+        for (int j = 0; j < nc; ++j) cn += lam_of(j) < B ? 1 : 0;
         if (cn < 1) cn = 1;
       }
       s_cnt = cn;
     }
-    for (int j = threadIdx.x; j < Ln; j += blockDim.x)
-      lv.lamP[P * Ln + j] = j < nc ? V[order[j] * nR + order[j]] : INFINITY;
+    for (int j = threadIdx.x; j < Ln; j += blockDim.x) lv.lamP[P * Ln + j] = j < nc ? lam_of(j) : INFINITY;
     __syncthreads();
     const int cn = s_cnt;
     // Psi (rows = eigenvectors), zero in unused rows and slots
     for (int idx = threadIdx.x; idx < Ln * nP; idx += blockDim.x) {
       const int j = idx / nP, i = idx % nP;
-      lv.Psi[(P * Ln + j) * nP + i] = (j < cn && cidx[i] >= 0) ? N[cidx[i] * nR + order[j]] : 0.0;
+      double v = 0.0;
+      if (j < cn && cidx[i] >= 0) v = direct ? Z[j * nR + cidx[i]] : N[cidx[i] * nR + order[j]];
+      lv.Psi[(P * Ln + j) * nP + i] = v;
     }
   } else if (threadIdx.x == 0) {
     int last = 0;
@@ -550,105 +568,181 @@ __global__ void k_add_null_shift(double* __restrict__ A, const double* __restric
   A[idx] += sigma * z[i] * z[j] / scal[0];
 }
 
-// Gauss-Jordan inversion in place (no pivoting: the matrix is symmetric positive
-// definite, shifted along its null vector when singular), kGjBlock pivots per pass
-// over the matrix, with the arithmetic of one pivot at a time.  Step k of the
-// single-pivot form: with c_i = A[i][k] / A[k][k] and r_j = A[k][j],
-//   A[i][j] = fma(-c_i, r_j, A[i][j]) for i, j != k,  A[k][j] = r_j / A[k][k],
-//   A[i][k] = -c_i,  A[k][k] = 1 / A[k][k].
-// For the pivots P = {k, .., k + b - 1} the first launch replays these b steps on
-// the rows and columns of P (thread j owns row P's entries in column j and column
-// P's entries in row j; every thread also replays the b x b pivot block) and
-// records each step's c and r; the second applies the b rank-1 updates to the
-// other entries in step order.  Every entry sees the same operations in the same
-// order as with one pivot per pass, so the bits are the same, with one sweep of
-// the matrix per b pivots instead of one per pivot (the 3740-unknown inverse of the
-// IMPES hierarchy: 224 ms with one pivot per pass).
-__global__ void k_gj_panel(const double* __restrict__ A, int64_t n, int64_t k, int b, double* __restrict__ cbuf,
-                           double* __restrict__ rbuf, double* __restrict__ rfin, double* __restrict__ cfin,
-                           double* __restrict__ ppfin, double* stats) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  double PP[kGjBlock][kGjBlock];
-#pragma unroll
-  for (int s = 0; s < kGjBlock; ++s)
-#pragma unroll
-    for (int u = 0; u < kGjBlock; ++u) PP[s][u] = (s < b && u < b) ? A[(k + s) * n + k + u] : 0.0;
-  const bool act = j < n && !(j >= k && j < k + b);
-  double R[kGjBlock], Cj[kGjBlock];
-#pragma unroll
-  for (int s = 0; s < kGjBlock; ++s) {
-    R[s] = (act && s < b) ? A[(k + s) * n + j] : 0.0;
-    Cj[s] = (act && s < b) ? A[j * n + k + s] : 0.0;
+// Inversion in place of the symmetric positive definite matrix (shifted along its null
+// vector when singular) by sweeping blocks of kGjBlock pivots: with P the block,
+// A[P, P] = L L^T, M = L^-1 and Y = A[:, P] M^T,
+//   A[i, j] -= Y_i Y_j^T (i, j not in P),  A[i, P] = Y_i M,  A[P, P] = -M^T M,
+// which leaves -A^-1 after the last block.  (With the explicit inverse of A[P, P] in
+// place of its factor the error grows with cond(A[P, P]) instead of its root.)  The matrix
+// stays symmetric, so only the lower triangle is kept: n^3 / 2 FMAs, which bind it (FP64:
+// two lanes per clock and SM; 3740 unknowns: 43 ms at that rate).  Two launches per block:
+// k_sweep_panel (every CTA factors the block for itself and forms kSwRows rows of Y and
+// Y M), k_sweep_update (a 64 x 64 tile of the lower triangle per CTA, 4 x 4 outputs per
+// thread: 410 us a block of 32, 395 at the FP64 rate).  Gauss-Jordan on the whole matrix
+// with four pivots per pass took 131 ms on the 3740 unknowns of the reservoir hierarchy,
+// this 53.
+constexpr int kSwTile = 64, kSwRows = 32;
+
+// Y[n][kGjBlock], C = Y M [n][kGjBlock] of the block at k (b pivots; columns beyond b zero);
+// D = M^T M (b x b) from the first CTA.  The lower triangle holds A.
+__global__ void __launch_bounds__(256) k_sweep_panel(const double* __restrict__ A, int64_t n, int64_t k, int b,
+                                                     double* __restrict__ Y, double* __restrict__ C,
+                                                     double* __restrict__ D, double* stats) {
+  constexpr int NB = kGjBlock;
+  __shared__ double d[NB][2 * NB + 1];               // [A | I], eliminated to [. | L^-1]
+  __shared__ double w[kSwRows][NB + 1], y[kSwRows][NB + 1];
+  __shared__ double s_r[NB];
+  const int tid = threadIdx.x;
+  const int64_t i0 = (int64_t)blockIdx.x * kSwRows;
+  for (int o = tid; o < NB * NB; o += 256) {
+    const int r = o / NB, c = o % NB;
+    d[r][c] = (r < b && c < b) ? (c <= r ? A[(k + r) * n + k + c] : A[(k + c) * n + k + r]) : (r == c ? 1.0 : 0.0);
+    d[r][NB + c] = r == c ? 1.0 : 0.0;
   }
-#pragma unroll
-  for (int t = 0; t < kGjBlock; ++t) {
-    if (t >= b) break;
-    const double piv = PP[t][t];
-    if (blockIdx.x == 0 && threadIdx.x == 0 && !(piv > 0.0)) atomic_max_pos(&stats[1], 1.0);
-    if (act) {
-      const double c = Cj[t] / piv, r = R[t];
-      cbuf[(int64_t)t * n + j] = c;
-      rbuf[(int64_t)t * n + j] = r;
-#pragma unroll
-      for (int s = 0; s < kGjBlock; ++s)
-        if (s < b && s != t) R[s] = fma(-(PP[s][t] / piv), r, R[s]);
-      R[t] = r / piv;
-#pragma unroll
-      for (int u = 0; u < kGjBlock; ++u)
-        if (u < b && u != t) Cj[u] = fma(-c, PP[t][u], Cj[u]);
-      Cj[t] = -c;
-    }
-    double cs[kGjBlock];
-#pragma unroll
-    for (int s = 0; s < kGjBlock; ++s) cs[s] = PP[s][t] / piv;
-#pragma unroll
-    for (int s = 0; s < kGjBlock; ++s)
-#pragma unroll
-      for (int u = 0; u < kGjBlock; ++u)
-        if (s < b && u < b && s != t && u != t) PP[s][u] = fma(-cs[s], PP[t][u], PP[s][u]);
-#pragma unroll
-    for (int u = 0; u < kGjBlock; ++u)
-      if (u < b && u != t) PP[t][u] = PP[t][u] / piv;
-#pragma unroll
-    for (int s = 0; s < kGjBlock; ++s)
-      if (s < b && s != t) PP[s][t] = -cs[s];
-    PP[t][t] = 1.0 / piv;
+  // the CTA's rows of A[:, P]: from the rows below the block, or the block's rows where i is before it
+  for (int o = tid; o < kSwRows * NB; o += 256) {
+    int r, c;
+    if (i0 + kSwRows <= k) { r = o % kSwRows; c = o / kSwRows; }    // A[k + c][i]: consecutive threads along i
+    else { r = o / NB; c = o % NB; }
+    const int64_t i = i0 + r;
+    double v = 0.0;
+    if (i < n && c < b) v = i >= k + c ? A[i * n + k + c] : A[(k + c) * n + i];
+    w[r][c] = v;
   }
-  if (act) {
+  __syncthreads();
+  // Step t subtracts row t / pivot from the rows below (columns beyond t of A, up to t of
+  // M); rows stay unscaled, s_r[t] = 1 / sqrt(pivot) scales them at the end.  Warp ry has the
+  // rows ry + 8 q, lane x column x of A or of M, so a step is one barrier; the pivot's root
+  // is taken by the lane that has just formed it.
+  const int x = tid & 31, ry = tid >> 5;
+  if (tid == 0) {
+    s_r[0] = rsqrt(d[0][0]);
+    if (blockIdx.x == 0 && !(d[0][0] > 0.0)) atomic_max_pos(&stats[1], 1.0);
+  }
+  __syncthreads();
+  for (int t = 0; t + 1 < b; ++t) {
+    const int c = x > t ? x : NB + x;
+    const double r = s_r[t], tv = d[t][c] * r;
 #pragma unroll
-    for (int s = 0; s < kGjBlock; ++s)
-      if (s < b) {
-        rfin[(int64_t)s * n + j] = R[s];
-        cfin[j * kGjBlock + s] = Cj[s];
+    for (int q = 0; q < NB / 8; ++q) {
+      const int i = ry + 8 * q;
+      if (i <= t) continue;
+      const double v = fma(-(d[i][t] * r), tv, d[i][c]);
+      d[i][c] = v;
+      if (i == t + 1 && x == t + 1) {
+        s_r[i] = rsqrt(v);
+        if (blockIdx.x == 0 && !(v > 0.0)) atomic_max_pos(&stats[1], 1.0);
       }
+    }
+    __syncthreads();
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0)
-    for (int s = 0; s < b; ++s)
-      for (int u = 0; u < b; ++u) ppfin[s * b + u] = PP[s][u];
+#pragma unroll
+  for (int q = 0; q < NB / 8; ++q) {
+    const int i = ry + 8 * q;
+    if (i < b) d[i][NB + x] *= s_r[i];
+  }
+  __syncthreads();
+  // D = M^T M
+  if (blockIdx.x == 0)
+    for (int o = tid; o < NB * NB; o += 256) {
+      const int r = o / NB, c = o % NB;
+      double v = 0.0;
+      for (int q = r > c ? r : c; q < NB; ++q) v = fma(d[q][NB + r], d[q][NB + c], v);
+      D[o] = v;
+    }
+  // Y = W M^T, C = Y M: thread = (row, every eighth column)
+  const int r = tid >> 3, c0 = tid & 7;
+#pragma unroll
+  for (int q = 0; q < NB / 8; ++q) {
+    const int c = c0 + 8 * q;
+    double v = 0.0;
+    for (int j = 0; j <= c; ++j) v = fma(w[r][j], d[c][NB + j], v);
+    y[r][c] = v;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NB / 8; ++q) {
+    const int c = c0 + 8 * q;
+    double v = 0.0;
+    for (int j = c; j < NB; ++j) v = fma(y[r][j], d[j][NB + c], v);
+    if (i0 + r < n) {
+      Y[(i0 + r) * NB + c] = c < b ? y[r][c] : 0.0;
+      C[(i0 + r) * NB + c] = c < b ? v : 0.0;
+    }
+  }
 }
 
-__global__ void k_gj_block_update(double* __restrict__ A, int64_t n, int64_t k, int b,
-                                  const double* __restrict__ cbuf, const double* __restrict__ rbuf,
-                                  const double* __restrict__ rfin, const double* __restrict__ cfin,
-                                  const double* __restrict__ ppfin) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * n) return;
-  const int64_t i = idx / n, j = idx % n;
-  const bool pi = i >= k && i < k + b, pj = j >= k && j < k + b;
-  double v;
-  if (pi && pj) {
-    v = ppfin[(i - k) * b + (j - k)];
-  } else if (pi) {
-    v = rfin[(i - k) * n + j];
-  } else if (pj) {
-    v = cfin[i * kGjBlock + (j - k)];
-  } else {
-    v = A[idx];
+__global__ void __launch_bounds__(256) k_sweep_update(double* __restrict__ A, int64_t n, int64_t k, int b,
+                                                      const double* __restrict__ Y, const double* __restrict__ C,
+                                                      const double* __restrict__ D) {
+  __shared__ double cs[kGjBlock][kSwTile + 1], ws[kGjBlock][kSwTile + 1];
+  // tile (ti, tj), tj <= ti, of the lower triangle
+  const unsigned t = blockIdx.x;
+  unsigned ti = (unsigned)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
+  while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+  while (ti * (ti + 1) / 2 > t) --ti;
+  const unsigned tj = t - ti * (ti + 1) / 2;
+  const int64_t i0 = (int64_t)ti * kSwTile, j0 = (int64_t)tj * kSwTile;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  double v[4][4];
 #pragma unroll
-    for (int t = 0; t < kGjBlock; ++t)
-      if (t < b) v = fma(-cbuf[(int64_t)t * n + i], rbuf[(int64_t)t * n + j], v);
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int64_t i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
+      v[r][c] = (i < n && j <= i) ? A[i * n + j] : 0.0;
+    }
+  for (int o = tid; o < kSwTile * kGjBlock; o += 256) {
+    const int r = o / kGjBlock, c = o % kGjBlock;
+    cs[c][r] = i0 + r < n ? -Y[(i0 + r) * kGjBlock + c] : 0.0;
+    ws[c][r] = j0 + r < n ? Y[(j0 + r) * kGjBlock + c] : 0.0;
   }
-  A[idx] = v;
+  __syncthreads();
+#pragma unroll 4
+  for (int q = 0; q < b; ++q) {
+    double a[4], w[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) a[r] = cs[q][ty + 16 * r];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) w[c] = ws[q][tx + 16 * c];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) v[r][c] = fma(a[r], w[c], v[r][c]);
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int64_t i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
+      if (i >= n || j > i) continue;
+      const bool pi = i >= k && i < k + b, pj = j >= k && j < k + b;
+      double o = v[r][c];
+      if (pi && pj) o = -D[(i - k) * kGjBlock + (j - k)];
+      else if (pj) o = C[i * kGjBlock + (j - k)];
+      else if (pi) o = C[j * kGjBlock + (i - k)];
+      A[i * n + j] = o;
+    }
+}
+
+// A <- -A from the lower triangle, both triangles
+__global__ void __launch_bounds__(256) k_sweep_finish(double* __restrict__ A, int64_t n) {
+  __shared__ double s[32][33];
+  const int64_t i0 = (int64_t)blockIdx.y * 32, j0 = (int64_t)blockIdx.x * 32;
+  if (j0 > i0) return;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  for (int r = y; r < 32; r += 8) {
+    const int64_t i = i0 + r, j = j0 + x;
+    s[r][x] = (i < n && j <= i) ? -A[i * n + j] : 0.0;
+  }
+  __syncthreads();
+  for (int r = y; r < 32; r += 8) {
+    const int64_t i = i0 + r, j = j0 + x;
+    if (i < n && j <= i) A[i * n + j] = s[r][x];
+    // entry (j0 + r, i0 + x) of the upper triangle
+    const int64_t iu = j0 + r, ju = i0 + x;
+    if (iu < n && ju < n && iu < ju) A[iu * n + ju] = s[x][r];
+  }
 }
 
 // w = B zhat (B the inverse), gamma = zhat^T w; zhat = z / |z|
@@ -746,30 +840,24 @@ void launch_level1_galerkin(msmg_ctx* c, cudaStream_t s, bool threshold) {
                                              l2.F, l2.z, l2.cnt, f.Wd);
 }
 
-int launch_coarse_setup(msmg_ctx* c, int l, cudaStream_t s) {
+static int coarse_setup(msmg_ctx* c, int l, bool given, cudaStream_t s) {
   CoarseLevel& lv = c->lev[l];
   CoarseLevel& nx = c->lev[l + 1];
   if (lv.nP > 96) return MSMG_ERR_UNSUPPORTED;
-  const size_t sm = jac_smem(lv.nP, 3);
+  size_t sm = jac_smem(lv.nP, 3);
+  int tri = given ? 0 : tri_doubles(lv.nP, lv.Lnext);
+  if (sm + (size_t)tri * sizeof(double) > 226 * 1024) tri = 0;
+  sm += (size_t)tri * sizeof(double);
   cudaFuncSetAttribute(k_coarse_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_coarse_setup<<<(unsigned)lv.mP, 256, sm, s>>>(lv, nx, c->dtmp, 0, c->opts.coarse_smoother == MSMG_BLOCK_IC0,
-                                                  c->opts.eig_threshold[l - 1]);
+  k_coarse_setup<<<(unsigned)lv.mP, 256, sm, s>>>(lv, nx, c->dtmp, given ? 1 : 0,
+                                                  c->opts.coarse_smoother == MSMG_BLOCK_IC0,
+                                                  given ? 0.0 : c->opts.eig_threshold[l - 1], tri);
   k_coarse_galerkin_off<<<(unsigned)lv.mP, 128, 0, s>>>(lv, nx);
   return 0;
 }
-
+int launch_coarse_setup(msmg_ctx* c, int l, cudaStream_t s) { return coarse_setup(c, l, false, s); }
 // Same with the bases Psi already in place (imported): no eigensolve.
-int launch_coarse_setup_given(msmg_ctx* c, int l, cudaStream_t s) {
-  CoarseLevel& lv = c->lev[l];
-  CoarseLevel& nx = c->lev[l + 1];
-  if (lv.nP > 96) return MSMG_ERR_UNSUPPORTED;
-  const size_t sm = jac_smem(lv.nP, 3);
-  cudaFuncSetAttribute(k_coarse_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  k_coarse_setup<<<(unsigned)lv.mP, 256, sm, s>>>(lv, nx, c->dtmp, 1, c->opts.coarse_smoother == MSMG_BLOCK_IC0,
-                                                  0.0);
-  k_coarse_galerkin_off<<<(unsigned)lv.mP, 128, 0, s>>>(lv, nx);
-  return 0;
-}
+int launch_coarse_setup_given(msmg_ctx* c, int l, cudaStream_t s) { return coarse_setup(c, l, true, s); }
 
 int launch_coarsest(msmg_ctx* c, cudaStream_t s) {
   CoarseLevel& lv = c->lev[c->nL];
@@ -798,12 +886,10 @@ int launch_coarsest(msmg_ctx* c, cudaStream_t s) {
   }
   const int64_t nk = lv.nk;
   double* B = c->dtmp + 16;
-  double* cbuf = B + n * n;                  // [kGjBlock][n] each step's multipliers
-  double* rbuf = cbuf + kGjBlock * n;         // [kGjBlock][n] each step's pivot row
-  double* rfin = rbuf + kGjBlock * n;         // [kGjBlock][n] the pivot rows after the pass
-  double* cfin = rfin + kGjBlock * n;         // [n][kGjBlock] the pivot columns after the pass
-  double* ppfin = cfin + kGjBlock * n;        // [kGjBlock^2] the pivot block after the pass
-  double* w = ppfin + kGjBlock * kGjBlock;
+  double* Yb = B + n * n;                    // [n][kGjBlock] the block's columns times its inverse factor
+  double* Cb = Yb + kGjBlock * n;             // [n][kGjBlock] times the block's inverse
+  double* Db = Cb + kGjBlock * n;             // [kGjBlock^2] that inverse
+  double* w = Db + kGjBlock * kGjBlock;
   double* scal = c->dtmp + 4;
   MSMG_CUDA_TRY(cudaMemsetAsync(B, 0, (size_t)n * n * sizeof(double), s));
   k_assemble_dense<<<(unsigned)lv.me, 64, 0, s>>>(lv, B);
@@ -816,17 +902,19 @@ int launch_coarsest(msmg_ctx* c, cudaStream_t s) {
     z = lv.pinv + nk * nk;
   }
   const unsigned g2 = (unsigned)((nk * nk + 255) / 256);
-  const unsigned g1 = (unsigned)((nk + 255) / 256);
   const bool singular = c->fine.Wd == nullptr;   // a cell term (wells) removes the null space
   if (singular) {
     k_coarsest_scalars<<<1, 256, 0, s>>>(B, z, nk, scal);
     k_add_null_shift<<<g2, 256, 0, s>>>(B, z, nk, scal);
   }
+  const int64_t nt = (nk + kSwTile - 1) / kSwTile;
   for (int64_t k = 0; k < nk; k += kGjBlock) {
     const int b = (int)(nk - k < kGjBlock ? nk - k : kGjBlock);
-    k_gj_panel<<<g1, 256, 0, s>>>(B, nk, k, b, cbuf, rbuf, rfin, cfin, ppfin, c->dtmp);
-    k_gj_block_update<<<g2, 256, 0, s>>>(B, nk, k, b, cbuf, rbuf, rfin, cfin, ppfin);
+    k_sweep_panel<<<(unsigned)((nk + kSwRows - 1) / kSwRows), 256, 0, s>>>(B, nk, k, b, Yb, Cb, Db, c->dtmp);
+    k_sweep_update<<<(unsigned)(nt * (nt + 1) / 2), 256, 0, s>>>(B, nk, k, b, Yb, Cb, Db);
   }
+  const unsigned n32 = (unsigned)((nk + 31) / 32);
+  k_sweep_finish<<<dim3(n32, n32), 256, 0, s>>>(B, nk);
   if (singular) {
     k_gemv_z<<<(unsigned)((nk * 32 + 255) / 256), 256, 0, s>>>(B, z, nk, scal, w);
     k_dot_zw<<<1, 256, 0, s>>>(z, w, nk, scal);
