@@ -402,10 +402,13 @@ int msmg_setup(const msmg_grid* grid, const void* kappa, int kappa_components, i
   cudaGetDevice(&c->device);
   cudaEventCreate(&c->ev0);
   cudaEventCreate(&c->ev1);
-  // untuned defaults: separate prolongation for single solves, fused for batches
-  c->tune_fused[0] = 0;
-  c->tune_fused[1] = 1;
-  c->tune_tail[0] = c->tune_tail[1] = 2;   // the fused coarse cycle, where the hierarchy allows it
+  // untuned defaults: separate prolongation and a launch per coarse step, the fastest of the
+  // variants on every hierarchy they were timed on (us per iteration, best / the fused
+  // prolongation / the cooperative coarse cycle: 32^3 FP64 76 / 78 / 91, 96^3 FP64
+  // 298 / 317 / 328, 256^3 mixed 1297 / 1351 / 1366, 60x220x85 with wells 423 / 501 / 477,
+  // 96^3 with 16 right-hand sides 969 / 1013 / 996)
+  c->tune_fused[0] = c->tune_fused[1] = 0;
+  c->tune_tail[0] = c->tune_tail[1] = 0;
   for (int k = 0; k < 3; ++k) cudaEventCreateWithFlags(&c->poll_evs[k], cudaEventDisableTiming);
   *out = c;
   // pinned host mirrors of the PCG scalars (latest + two in-flight chunks),
