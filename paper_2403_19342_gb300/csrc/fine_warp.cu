@@ -1,7 +1,8 @@
-// Fine-level PCG iteration kernels, one warp per element (two in the FP64 k_post
-// on 8^3 elements, see elem_threads).
+// Fine-level PCG iteration kernels.  Two sets: one warp per element (two in the FP64
+// k_post on 8^3 elements, see elem_threads), which 8^3 elements and small FP64 grids
+// take, and groups of elements per CTA (the k_*_grp kernels, use_groups) for the rest.
 //
-// Each element of E_1 (bx x by x bz cells) is handled by one warp.  Its data is
+// In the first set each element of E_1 (bx x by x bz cells) is handled by one warp.  Its data is
 // one contiguous chunk of every block-major array; the warp stages what it
 // reuses (the iterate u with its one-cell face halo, the face coefficients T,
 // the inverse IC(0) pivots) in shared memory with asynchronous copies, all in
@@ -60,6 +61,10 @@ template <typename G>
 struct IsCube8 : std::false_type {};
 template <>
 struct IsCube8<GeoC<8, 8, 8>> : std::true_type {};
+template <typename G>
+struct IsGeoC : std::false_type {};
+template <int BX, int BY, int BZ>
+struct IsGeoC<GeoC<BX, BY, BZ>> : std::true_type {};
 
 // Threads per element of the staged kernels: two warps for an 8^3 element in
 // the FP64 k_post (a wavefront has at most 48 cells, so each thread takes at
@@ -1332,6 +1337,720 @@ __global__ void __launch_bounds__(kPmWarps * 32, kPmCtasPerSm) k_pmatvec(const d
   });
 }
 
+// ------------------------------------------------------------------ groups of elements
+// The fine kernels on groups of consecutive elements, E per CTA of 128 threads (E by <=
+// 32), for elements smaller than 8^3 (use_groups).  Latency and issue bind them.  The
+// group's cells are one contiguous range of every array, which all threads stream (a warp
+// per 80-cell element left lanes idle and its unrolled loops mostly predicated off); the
+// IC(0) sweeps are run by one warp, a lane per (element, ly): lane (e, ly) walks its
+// x-lines lz = 0 .. bz-1, one per step s = ly + lz, keeping the line in registers.  The line's neighbours are its own previous line (lz - 1) and the previous line
+// of the lane before it (ly - 1, by shuffle), so a sweep of an 8^3 element is 15 steps of
+// 8 cells without a barrier, and reads shared memory in 16-byte pieces: 14 instructions a
+// step for four elements.  Per cell the arithmetic and its order are those of w_ic0_s.
+// 60 x 220 x 85 cells, 4 x 4 x 5 elements, mixed (event times, us): pre 76 -> 39, post
+// 132 -> 56, restrict 61 -> 47, pmatvec 65 -> 48.  On 8^3 elements the same kernels are
+// slower than a warp per element (128^3: post 63 against 51; 256^3: pre 279 against 262:
+// the sweeping warp's chains are four times longer and the rest of the CTA waits for
+// them), so those keep theirs.
+// Shared memory holds the planes of an element PP apart (a multiple of 32 words gets 4
+// more: lanes of one element are then on different banks), elements EP = PP bz apart.
+constexpr int kGThreads = 128;
+constexpr int kGCells = 16;                    // cells per thread: E nb <= 2048
+
+struct Grp {
+  int E, PP, EP;
+};
+template <typename G>
+__host__ __device__ constexpr Grp make_grp(const G& g) {
+  Grp q{};
+  const int e1 = 32 / g.by, e2 = kGCells * kGThreads / g.nb;
+  q.E = e1 < e2 ? e1 : e2;
+  if (q.E > 16) q.E = 16;
+  q.PP = g.bx * g.by + (g.bx * g.by % 32 == 0 ? 4 : 0);
+  q.EP = q.PP * g.bz;
+  return q;
+}
+template <typename G>
+__host__ __device__ inline int grp_pre_floats(const G& g) {
+  const Grp q = make_grp(g);
+  return 5 * r4(q.E * q.EP);
+}
+template <typename G>
+__host__ __device__ inline int grp_post_floats(const G& g) {
+  const Grp q = make_grp(g);
+  return r4(q.E * r4(g.P)) + 4 * r4(q.E * q.EP) + q.E * (r4(g.by * g.bz) + r4(g.bx * g.bz) + r4(g.bx * g.by));
+}
+
+// t0, t1, t2, dinv of elements e0 .. e0 + ne - 1 into dst (four arrays r4(E EP) apart): bulk
+// copies on the mbarrier where the sizes allow (returns true: wait for phase 0), per-thread
+// copies otherwise.  Run by the whole CTA; ends with a CTA barrier in the bulk case.
+template <typename V, typename G>
+__device__ __forceinline__ bool grp_stage(V* dst, const V* __restrict__ T, const V* __restrict__ invd, int64_t n, int64_t e0, int ne, const G& g, const Grp& q, unsigned bar) {
+  const int stride = r4(q.E * q.EP), plane = g.bx * g.by;
+  const bool packed = q.PP == plane;
+  const int64_t base = e0 * g.nb;
+  constexpr int per = 16 / sizeof(V);                // values of a 16-byte piece
+  const bool bulk = n % per == 0 && (packed ? (q.E * g.nb) % per == 0 && (ne * g.nb) % per == 0
+                                            : plane % per == 0 && q.PP % per == 0);
+  if (bulk) {
+    if (threadIdx.x == 0) {
+      mbar_init(bar, 1);
+      mbar_expect_tx(bar, (unsigned)(4 * ne * g.nb * sizeof(V)));
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      if (packed) {
+        const int a = threadIdx.x;
+        if (a < 4) {
+          const V* src = a < 3 ? T + (int64_t)a * n + base : invd + base;
+          bulk_g2s(dst + a * stride, src, (unsigned)(ne * g.nb * sizeof(V)), bar);
+        }
+      } else {
+        for (int k = threadIdx.x; k < 4 * ne * g.bz; k += 32) {
+          const int a = k & 3, ep = k >> 2;              // ep: plane of the group
+          const V* src = (a < 3 ? T + (int64_t)a * n + base : invd + base) + (int64_t)ep * plane;
+          bulk_g2s(dst + a * stride + ep * q.PP, src, (unsigned)(plane * sizeof(V)), bar);
+        }
+      }
+    }
+    return true;
+  }
+  for (int a = 0; a < 4; ++a) {
+    const V* src = a < 3 ? T + (int64_t)a * n + base : invd + base;
+    for (int k = threadIdx.x; k < ne * g.nb; k += kGThreads) {
+      const int ep = k / plane;
+      cp_async_elem(dst + a * stride + ep * q.PP + (k - ep * plane), src + k);
+    }
+  }
+  return false;
+}
+// the group's staged copies have landed (all threads; also a CTA barrier)
+__device__ __forceinline__ bool grp_landed(bool bulk, unsigned bar, PcgScalars* sc, int* err) {
+  cp_async_wait_all();
+  const bool ok = __syncthreads_and(!bulk || mbar_wait(bar, 0)) != 0;
+  if (!ok) {
+    if (threadIdx.x == 0) {
+      atomicExch(err, 1);
+      if (sc) sc->done = 2;
+    }
+    mbar_wait(bar, 0);
+    __syncthreads();
+  }
+  return ok;
+}
+
+// a line of N floats from and to shared memory
+template <int N, typename V>
+__device__ __forceinline__ void ld_line(V (&v)[N], const V* p) {
+  if constexpr (N % 4 == 0 && sizeof(V) == 4) {
+#pragma unroll
+    for (int k = 0; k < N / 4; ++k) {
+      const float4 t = *reinterpret_cast<const float4*>(p + 4 * k);
+      v[4 * k] = t.x; v[4 * k + 1] = t.y; v[4 * k + 2] = t.z; v[4 * k + 3] = t.w;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = p[k];
+  }
+}
+template <int N, typename V>
+__device__ __forceinline__ void st_line(V* p, const V (&v)[N]) {
+  if constexpr (N % 4 == 0 && sizeof(V) == 4) {
+#pragma unroll
+    for (int k = 0; k < N / 4; ++k)
+      *reinterpret_cast<float4*>(p + 4 * k) = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < N; ++k) p[k] = v[k];
+  }
+}
+
+// y <- M^{-1} y for the group, by one warp; lines of BX cells in registers.  d: t0, t1, t2, dinv.
+template <int BX, typename V, typename G>
+__device__ __forceinline__ void grp_ic0_lines(const V* d, V* y, const G& g, const Grp& q, int ne) {
+  const int stride = r4(q.E * q.EP);
+  const V *t0 = d, *t1 = d + stride, *t2 = d + 2 * stride, *di = d + 3 * stride;
+  const int lane = threadIdx.x & 31, el = lane / g.by, ly = lane - el * g.by;
+  const bool on = el < ne && el < q.E;
+  const int base = on ? el * q.EP + ly * BX : 0;
+  const int top = g.by + g.bz - 2;
+  const bool ym = ly > 0, yp = ly + 1 < g.by;
+  V last[BX];                              // this lane's previous line
+#pragma unroll
+  for (int x = 0; x < BX; ++x) last[x] = (V)0;
+  for (int s = 0; s <= top; ++s) {
+    V nb[BX];                              // line (ly - 1, lz), the lane before's last
+#pragma unroll
+    for (int x = 0; x < BX; ++x) nb[x] = __shfl_up_sync(0xffffffffu, last[x], 1);
+    const int lz = s - ly;
+    if (on && lz >= 0 && lz < g.bz) {
+      const int o = base + lz * q.PP;
+      V v[BX], a0[BX], a1[BX], a2[BX], w[BX];
+      ld_line<BX>(v, y + o);
+      ld_line<BX>(a0, t0 + o);
+      ld_line<BX>(a1, t1 + (ym ? o - BX : o));
+      ld_line<BX>(a2, t2 + (lz > 0 ? o - q.PP : o));
+      ld_line<BX>(w, di + o);
+#pragma unroll
+      for (int x = 0; x < BX; ++x) {
+        V acc = v[x];
+        if (x > 0) acc = fma(a0[x - 1], v[x - 1], acc);
+        if (ym) acc = fma(a1[x], nb[x], acc);
+        if (lz > 0) acc = fma(a2[x], last[x], acc);
+        v[x] = acc * w[x];
+      }
+#pragma unroll
+      for (int x = 0; x < BX; ++x) last[x] = v[x];
+      st_line<BX>(y + o, v);
+    }
+  }
+  for (int s = top; s >= 0; --s) {
+    V nb[BX];                              // line (ly + 1, lz), the lane after's last
+#pragma unroll
+    for (int x = 0; x < BX; ++x) nb[x] = __shfl_down_sync(0xffffffffu, last[x], 1);
+    const int lz = s - ly;
+    if (on && lz >= 0 && lz < g.bz) {
+      const int o = base + lz * q.PP;
+      V v[BX], a0[BX], a1[BX], a2[BX], w[BX];
+      ld_line<BX>(v, y + o);
+      ld_line<BX>(a0, t0 + o);
+      ld_line<BX>(a1, t1 + o);
+      ld_line<BX>(a2, t2 + o);
+      ld_line<BX>(w, di + o);
+      const bool zp = lz + 1 < g.bz;
+#pragma unroll
+      for (int x = BX - 1; x >= 0; --x) {
+        V acc = (V)0;
+        if (x + 1 < BX) acc = fma(a0[x], v[x + 1], acc);
+        if (yp) acc = fma(a1[x], nb[x], acc);
+        if (zp) acc = fma(a2[x], last[x], acc);
+        v[x] = fma(w[x], acc, v[x]);
+      }
+#pragma unroll
+      for (int x = 0; x < BX; ++x) last[x] = v[x];
+      st_line<BX>(y + o, v);
+    }
+  }
+}
+// the same for any line length, cell by cell out of shared memory
+template <typename V, typename G>
+__device__ __forceinline__ void grp_ic0_any(const V* d, V* y, const G& g, const Grp& q, int ne) {
+  const int stride = r4(q.E * q.EP);
+  const V *t0 = d, *t1 = d + stride, *t2 = d + 2 * stride, *di = d + 3 * stride;
+  const int lane = threadIdx.x & 31, el = lane / g.by, ly = lane - el * g.by;
+  const bool on = el < ne && el < q.E;
+  const int base = on ? el * q.EP + ly * g.bx : 0;
+  const int top = g.by + g.bz - 2;
+  for (int s = 0; s <= top; ++s) {
+    const int lz = s - ly;
+    if (on && lz >= 0 && lz < g.bz) {
+      V prev = (V)0;
+      for (int x = 0; x < g.bx; ++x) {
+        const int c = base + lz * q.PP + x;
+        V acc = y[c];
+        if (x > 0) acc = fma(t0[c - 1], prev, acc);
+        if (ly > 0) acc = fma(t1[c - g.bx], y[c - g.bx], acc);
+        if (lz > 0) acc = fma(t2[c - q.PP], y[c - q.PP], acc);
+        prev = acc * di[c];
+        y[c] = prev;
+      }
+    }
+    __syncwarp();
+  }
+  for (int s = top; s >= 0; --s) {
+    const int lz = s - ly;
+    if (on && lz >= 0 && lz < g.bz) {
+      V prev = (V)0;
+      for (int x = g.bx - 1; x >= 0; --x) {
+        const int c = base + lz * q.PP + x;
+        V acc = (V)0;
+        if (x + 1 < g.bx) acc = fma(t0[c], prev, acc);
+        if (ly + 1 < g.by) acc = fma(t1[c], y[c + g.bx], acc);
+        if (lz + 1 < g.bz) acc = fma(t2[c], y[c + q.PP], acc);
+        prev = fma(di[c], acc, y[c]);
+        y[c] = prev;
+      }
+    }
+    __syncwarp();
+  }
+}
+// one warp of the CTA sweeps (a different one from CTA to CTA: the SM's schedulers share
+// the work); starts and ends with a CTA barrier
+template <typename V, typename G>
+__device__ __forceinline__ void grp_ic0(const V* d, V* y, const G& g, const Grp& q, int ne) {
+  __syncthreads();
+  if ((threadIdx.x >> 5) == (blockIdx.x & 3)) {
+    if constexpr (IsGeoC<G>::value) {
+      grp_ic0_lines<G::bx>(d, y, g, q, ne);
+    } else {
+      if (g.bx == 4) grp_ic0_lines<4>(d, y, g, q, ne);
+      else if (g.bx == 6) grp_ic0_lines<6>(d, y, g, q, ne);
+      else if (g.bx == 8 && q.PP % 4 == 0) grp_ic0_lines<8>(d, y, g, q, ne);
+      else grp_ic0_any(d, y, g, q, ne);
+    }
+  }
+  __syncthreads();
+}
+
+// k_pre on groups: x += alpha p, r -= alpha q, r.r; rv = r in FP32, u = M^{-1} rv.
+template <typename V, typename G>
+__global__ void __launch_bounds__(kGThreads)
+    k_pre_grp(double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
+              const double* __restrict__ q, const V* __restrict__ T, const V* __restrict__ invd,
+              V* __restrict__ rv, V* __restrict__ u, int64_t n, G g, int64_t m, int update, RedSlot red,
+              PcgScalars* sc, int* err, int R) {
+  const BatchIdx bi = batch_idx(R);
+  if (sc) sc += bi.r;
+  if (sc && sc->done) return;
+  {
+    const int64_t off = (int64_t)bi.r * n;
+    x += off; r += off; p += off; q += off; rv += off; u += off;
+  }
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(8) unsigned long long s_bar;
+  const Grp gq = make_grp(g);
+  V* d = reinterpret_cast<V*>(smem);
+  V* y = d + 4 * r4(gq.E * gq.EP);
+  const unsigned bar = (unsigned)__cvta_generic_to_shared(&s_bar);
+  const int64_t e0 = (int64_t)bi.blk * gq.E, base = e0 * g.nb;
+  const int ne = m - e0 < gq.E ? (int)(m - e0) : gq.E;
+  const int cells = ne * g.nb, plane = g.bx * g.by;
+  const bool bulk = grp_stage(d, T, invd, n, e0, ne, g, gq, bar);
+  const double alpha = update ? sc->alpha : 0.0;
+  double acc = 0.0;
+  // batches of kB cells per thread: all loads of a batch are issued before use
+  constexpr int kB = 8;
+  for (int b0 = 0; b0 < cells; b0 += kB * kGThreads) {
+    double rr[kB], qq[kB], xx[kB], pp[kB];
+#pragma unroll
+    for (int i = 0; i < kB; ++i) {
+      const int c = b0 + kGThreads * i + (int)threadIdx.x;
+      const bool in = c < cells;
+      rr[i] = in ? r[base + c] : 0.0;
+      qq[i] = (in && update) ? q[base + c] : 0.0;
+      xx[i] = (in && update) ? x[base + c] : 0.0;
+      pp[i] = (in && update) ? p[base + c] : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < kB; ++i) {
+      const int c = b0 + kGThreads * i + (int)threadIdx.x;
+      if (c >= cells) continue;
+      double rc = rr[i];
+      if (update) {
+        x[base + c] = fma(alpha, pp[i], xx[i]);
+        rc = fma(-alpha, qq[i], rc);
+        r[base + c] = rc;
+        acc = fma(rc, rc, acc);
+      }
+      V fv;
+      if constexpr (sizeof(V) == 4) fv = f32_of_f64_rn(rc);   // integer pipes
+      else fv = rc;
+      const int ep = c / plane;
+      y[ep * gq.PP + (c - ep * plane)] = fv;
+      rv[base + c] = fv;
+    }
+  }
+  if (grp_landed(bulk, bar, sc, err)) {
+    grp_ic0(d, y, g, gq, ne);
+    for (int c = threadIdx.x; c < cells; c += kGThreads) {
+      const int ep = c / plane;
+      u[base + c] = y[ep * gq.PP + (c - ep * plane)];
+    }
+  }
+  if (update) {
+    double v[1] = {acc};
+    grid_reduce_r<1>(v, red, bi, [=] __device__(double* t) {
+      sc->rr = t[0];
+      sc->iter += 1;
+      if (sc->done != 0) return;   // a warp of this launch already stopped the solve
+      if (!isfinite(t[0])) sc->done = 2;
+      else if (t[0] <= sc->tol2) sc->done = 1;
+      else if (sc->iter >= sc->max_iter) sc->done = 3;
+    });
+  }
+}
+
+// k_post on groups: z = u' + M^{-1} (f - A u'), u' = u or, fused, u + Phi e_c; r.z and z.q.
+// y takes the place of the u tile once the residuals are formed.
+template <typename V, typename G, bool FUSE, int KC>
+__global__ void __launch_bounds__(kGThreads)
+    k_post_grp(const V* __restrict__ f, const double* __restrict__ r, const V* __restrict__ u,
+               const V* __restrict__ T, const V* __restrict__ Wd, const V* __restrict__ invd,
+               const V* __restrict__ Phi, const V* __restrict__ ec, int L, int64_t nc, double* __restrict__ z,
+               const double* __restrict__ qv, int64_t n, G g, int64_t m, const int* __restrict__ nbr, RedSlot red,
+               PcgScalars* sc, int* err, int R, int pf) {
+  const BatchIdx bi = batch_idx(R);
+  if (sc) sc += bi.r;
+  if (sc && sc->done) return;
+  {
+    const int64_t off = (int64_t)bi.r * n;
+    f += off; r += off; u += off; z += off;
+    if (qv) qv += off;
+    ec += (int64_t)bi.r * nc;
+  }
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ __align__(8) unsigned long long s_bar;
+  const Grp gq = make_grp(g);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tile = r4(g.P), stride = r4(gq.E * gq.EP), plane = g.bx * g.by;
+  const int n0 = r4(g.by * g.bz), n1 = r4(g.bx * g.bz), n2 = r4(g.bx * g.by);
+  V* ut = reinterpret_cast<V*>(smem);
+  V* y = ut;
+  V* d = ut + r4(gq.E * tile);
+  V* tm = d + 4 * stride;
+  const unsigned bar = (unsigned)__cvta_generic_to_shared(&s_bar);
+  const int64_t e0 = (int64_t)bi.blk * gq.E, base = e0 * g.nb;
+  const int ne = m - e0 < gq.E ? (int)(m - e0) : gq.E;
+  const int cells = ne * g.nb;
+  for (int el = warp; el < ne; el += kGThreads / 32) {
+    const WElem E = w_elem(e0 + el, nbr, g);
+    V* t = ut + el * tile;
+    w_cp_padded(t, u + E.base, g, lane);
+    w_cp_halo(t, u, E, g, lane);
+    V* q0 = tm + el * (n0 + n1 + n2);
+    w_cp_tminus(q0, q0 + n0, q0 + n0 + n1, T, n, E, g, lane);
+  }
+  const bool bulk = grp_stage(d, T, invd, n, e0, ne, g, gq, bar);
+  double v[2] = {0.0, 0.0};
+  if (grp_landed(bulk, bar, sc, err)) {
+    if (pf > 0 && threadIdx.x == 0 && n % 4 == 0 && (gq.E * g.nb) % 4 == 0) {
+      // the group one resident grid ahead into L2 (batched launches: many waves)
+      const unsigned b = blockIdx.x + (unsigned)pf;
+      if (b < gridDim.x) {
+        const int r2 = (int)(b % (unsigned)R);
+        const int64_t e2 = (int64_t)(b / (unsigned)R) * gq.E;
+        if (e2 + gq.E <= m) {
+          const unsigned bv = (unsigned)(gq.E * g.nb * sizeof(V)), bd = (unsigned)(gq.E * g.nb * sizeof(double));
+          const int64_t b2 = e2 * g.nb, o2 = (int64_t)(r2 - bi.r) * n + b2;
+          l2_prefetch(T + b2, bv);
+          l2_prefetch(T + n + b2, bv);
+          l2_prefetch(T + 2 * n + b2, bv);
+          l2_prefetch(invd + b2, bv);
+          l2_prefetch(u + o2, bv);
+          l2_prefetch(f + o2, bv);
+          if (sc) l2_prefetch(r + o2, bd);
+          if (qv) l2_prefetch(qv + o2, bd);
+          if (FUSE) l2_prefetch(Phi + b2 * L, bv * (unsigned)L);
+        }
+      }
+    }
+    if (FUSE) {
+      for (int el = warp; el < ne; el += kGThreads / 32)
+        w_prolong_tile<32>(ut + el * tile, Phi, ec, L, e0 + el, w_elem(e0 + el, nbr, g), g, lane);
+      __syncthreads();
+    }
+    V res[KC], uc[KC];
+#pragma unroll
+    for (int i = 0; i < KC; ++i) {
+      const int k = threadIdx.x + kGThreads * i;
+      res[i] = k < cells ? __ldg(f + base + k) : (V)0;
+    }
+    const V *t0 = d, *t1 = d + stride, *t2 = d + 2 * stride;
+    const int sy = g.bx + 2, sz = (g.bx + 2) * (g.by + 2);
+#pragma unroll
+    for (int i = 0; i < KC; ++i) {
+      const int k = threadIdx.x + kGThreads * i;
+      uc[i] = (V)0;
+      if (k >= cells) continue;
+      const int el = k / g.nb, c = k - el * g.nb;
+      const int lx = c % g.bx, t = c / g.bx, ly = t % g.by, lz = t / g.by;
+      const V* up = ut + el * tile + wpad(g, lx, ly, lz);
+      const int o = el * gq.EP + lz * gq.PP + g.bx * ly + lx;
+      const V* q0 = tm + el * (n0 + n1 + n2);
+      const V c0 = up[0];
+      const V mx = lx > 0 ? t0[o - 1] : q0[ly + g.by * lz];
+      const V my = ly > 0 ? t1[o - g.bx] : q0[n0 + lx + g.bx * lz];
+      const V mz = lz > 0 ? t2[o - gq.PP] : q0[n0 + n1 + lx + g.bx * ly];
+      V a = t0[o] * (c0 - up[1]) + mx * (c0 - up[-1]);
+      a += t1[o] * (c0 - up[sy]) + my * (c0 - up[-sy]);
+      a += t2[o] * (c0 - up[sz]) + mz * (c0 - up[-sz]);
+      a += Wd ? __ldg(Wd + base + k) * c0 : (V)0;
+      res[i] -= a;
+      uc[i] = c0;
+    }
+    // r and q are needed only after the sweeps: their loads overlap them
+    double rr[KC], qq[KC];
+#pragma unroll
+    for (int i = 0; i < KC; ++i) {
+      const int k = threadIdx.x + kGThreads * i;
+      const bool in = k < cells;
+      rr[i] = (in && sc) ? __ldg(r + base + k) : 0.0;
+      qq[i] = (in && qv) ? __ldg(qv + base + k) : 0.0;
+    }
+    __syncthreads();                           // every thread is done with the u tile
+#pragma unroll
+    for (int i = 0; i < KC; ++i) {
+      const int k = threadIdx.x + kGThreads * i;
+      if (k >= cells) continue;
+      const int ep = k / plane;
+      y[ep * gq.PP + (k - ep * plane)] = res[i];
+    }
+    grp_ic0(d, y, g, gq, ne);
+#pragma unroll
+    for (int i = 0; i < KC; ++i) {
+      const int k = threadIdx.x + kGThreads * i;
+      if (k >= cells) continue;
+      const int ep = k / plane;
+      const V zv = uc[i] + y[ep * gq.PP + (k - ep * plane)];
+      double zc;
+      if constexpr (sizeof(V) == 4) zc = f64_of_f32(zv);   // integer pipes
+      else zc = zv;
+      z[base + k] = zc;
+      v[0] = fma(rr[i], zc, v[0]);
+      v[1] = fma(zc, qq[i], v[1]);
+    }
+  }
+  if (sc) {
+    grid_reduce_r<2>(v, red, bi, [=] __device__(double* t) {
+      sc->rz_old = sc->rz;
+      sc->rz = t[0];
+      if (sc->flexible) sc->beta = sc->rz_old != 0.0 ? -sc->alpha * t[1] / sc->rz_old : 0.0;
+      else sc->beta = sc->rz_old != 0.0 ? t[0] / sc->rz_old : 0.0;
+      if (!isfinite(t[0])) sc->done = 2;
+    });
+  }
+}
+
+// Element bases of the group's neighbours (cells; -1: none) into shared memory, nb[el * 6 + f].
+template <typename G>
+__device__ __forceinline__ void grp_neighbours(int64_t* nb, const int* __restrict__ nbr, int64_t e0, int ne, const G& g) {
+  for (int k = threadIdx.x; k < 6 * ne; k += kGThreads) {
+    const int b = __ldg(nbr + e0 * 6 + k);
+    nb[k] = b >= 0 ? (int64_t)b * g.nb : -1;
+  }
+}
+// a cell of the group: its element, place in it and place in the element's padded tile
+struct GCell {
+  int el, c, lx, ly, lz, pc;
+};
+template <typename G>
+__device__ __forceinline__ GCell grp_cell(int k, const G& g) {
+  GCell q;
+  q.el = k / g.nb;
+  q.c = k - q.el * g.nb;
+  const int t = q.c / g.bx;
+  q.lx = q.c - t * g.bx;
+  q.lz = t / g.by;
+  q.ly = t - q.lz * g.by;
+  q.pc = wpad(g, q.lx, q.ly, q.lz);
+  return q;
+}
+// coefficient of the -d face of a cell: in the element, or held by the -d neighbour
+template <typename V, typename G>
+__device__ __forceinline__ V grp_tminus(const V* __restrict__ Td, int d, int64_t base, const int64_t* nb, const GCell& q,
+                                        const G& g) {
+  const int l = d == 0 ? q.lx : (d == 1 ? q.ly : q.lz), st = d == 0 ? 1 : (d == 1 ? g.bx : g.bx * g.by);
+  const int bd = d == 0 ? g.bx : (d == 1 ? g.by : g.bz);
+  if (l > 0) return __ldg(Td + base + q.el * g.nb + q.c - st);
+  const int64_t b = nb[q.el * 6 + 2 * d];
+  return b >= 0 ? __ldg(Td + b + q.c + (bd - 1) * st) : (V)0;
+}
+
+// k_restrict on groups: the residual a cell per thread and batch, then one warp sum per
+// (element, eigenvector) in the order of k_restrict.
+template <typename V, typename BT, typename G>
+__global__ void __launch_bounds__(kGThreads)
+    k_restrict_grp(const V* __restrict__ f, const V* __restrict__ u, const V* __restrict__ T, const V* __restrict__ Wd,
+                   const BT* __restrict__ Phi, int L, double* __restrict__ rc, int64_t nc, int64_t n, G g, int64_t m,
+                   const int* __restrict__ nbr, const PcgScalars* sc, int R) {
+  const BatchIdx bi = batch_idx(R);
+  if (sc) sc += bi.r;
+  if (sc && sc->done) return;
+  f += (int64_t)bi.r * n;
+  u += (int64_t)bi.r * n;
+  rc += (int64_t)bi.r * nc;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const Grp gq = make_grp(g);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tile = r4(g.P);
+  int64_t* nb = reinterpret_cast<int64_t*>(smem);
+  V* ut = reinterpret_cast<V*>(nb + 6 * gq.E);
+  V* w = ut + gq.E * tile;
+  const int64_t e0 = (int64_t)bi.blk * gq.E, base = e0 * g.nb;
+  const int ne = m - e0 < gq.E ? (int)(m - e0) : gq.E;
+  const int cells = ne * g.nb;
+  grp_neighbours(nb, nbr, e0, ne, g);
+  for (int el = warp; el < ne; el += kGThreads / 32) {
+    const WElem E = w_elem(e0 + el, nbr, g);
+    w_cp_padded(ut + el * tile, u + E.base, g, lane);
+    w_cp_halo(ut + el * tile, u, E, g, lane);
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  const int sy = g.bx + 2, sz = (g.bx + 2) * (g.by + 2);
+  constexpr int kB = 3;
+  for (int b0 = 0; b0 < cells; b0 += kB * kGThreads) {
+    V fv[kB], t0[kB], t1[kB], t2[kB], mx[kB], my[kB], mz[kB], wd[kB];
+    GCell q[kB];
+#pragma unroll
+    for (int i = 0; i < kB; ++i) {
+      const int k = b0 + kGThreads * i + (int)threadIdx.x;
+      if (k >= cells) continue;
+      q[i] = grp_cell(k, g);
+      fv[i] = __ldg(f + base + k);
+      t0[i] = __ldg(T + base + k);
+      t1[i] = __ldg(T + n + base + k);
+      t2[i] = __ldg(T + 2 * n + base + k);
+      mx[i] = grp_tminus(T, 0, base, nb, q[i], g);
+      my[i] = grp_tminus(T + n, 1, base, nb, q[i], g);
+      mz[i] = grp_tminus(T + 2 * n, 2, base, nb, q[i], g);
+      wd[i] = Wd ? __ldg(Wd + base + k) : (V)0;
+    }
+#pragma unroll
+    for (int i = 0; i < kB; ++i) {
+      const int k = b0 + kGThreads * i + (int)threadIdx.x;
+      if (k >= cells) continue;
+      const V* up = ut + q[i].el * tile + q[i].pc;
+      const V uc = up[0];
+      V a = t0[i] * (uc - up[1]) + mx[i] * (uc - up[-1]);
+      a += t1[i] * (uc - up[sy]) + my[i] * (uc - up[-sy]);
+      a += t2[i] * (uc - up[sz]) + mz[i] * (uc - up[-sz]);
+      if (Wd) a += wd[i] * uc;
+      w[k] = fv[i] - a;
+    }
+  }
+  __syncthreads();
+  for (int j = warp; j < ne * L; j += kGThreads / 32) {
+    const BT* ph = Phi + (e0 * L + j) * g.nb;
+    const V* we = w + j / L * g.nb;
+    V acc = (V)0;
+#pragma unroll 4
+    for (int c = lane; c < g.nb; c += 32) acc += (V)__ldg(ph + c) * we[c];
+    acc = warp_sum_t(acc);
+    if (lane == 0) rc[e0 * L + j] = (double)acc;
+  }
+}
+
+// k_pmatvec on groups: p = z + beta p_old on the cells and the face halos, q = A p, p.q.
+template <typename G>
+__global__ void __launch_bounds__(kGThreads)
+    k_pmatvec_grp(const double* __restrict__ z, const double* __restrict__ pold, double* __restrict__ pnew,
+                  double* __restrict__ qo, const double* __restrict__ T, const double* __restrict__ Dg, int64_t n, G g,
+                  int64_t m, const int* __restrict__ nbr, RedSlot red, PcgScalars* sc, int R) {
+  const BatchIdx bi = batch_idx(R);
+  sc += bi.r;
+  if (sc->done) return;
+  {
+    const int64_t off = (int64_t)bi.r * n;
+    z += off; pold += off; pnew += off; qo += off;
+  }
+  extern __shared__ __align__(16) unsigned char smem[];
+  const Grp gq = make_grp(g);
+  const int tile = r4(g.P);
+  int64_t* nb = reinterpret_cast<int64_t*>(smem);
+  double* ut = reinterpret_cast<double*>(nb + 6 * gq.E);
+  const int64_t e0 = (int64_t)bi.blk * gq.E, base = e0 * g.nb;
+  const int ne = m - e0 < gq.E ? (int)(m - e0) : gq.E;
+  const int cells = ne * g.nb;
+  grp_neighbours(nb, nbr, e0, ne, g);
+  const double beta = sc->beta;
+  constexpr int kB = 4;
+  for (int b0 = 0; b0 < cells; b0 += kB * kGThreads) {
+    double zz[kB], po[kB];
+#pragma unroll
+    for (int i = 0; i < kB; ++i) {
+      const int k = b0 + kGThreads * i + (int)threadIdx.x;
+      zz[i] = k < cells ? __ldg(z + base + k) : 0.0;
+      po[i] = k < cells ? __ldg(pold + base + k) : 0.0;
+    }
+#pragma unroll
+    for (int i = 0; i < kB; ++i) {
+      const int k = b0 + kGThreads * i + (int)threadIdx.x;
+      if (k >= cells) continue;
+      const GCell q = grp_cell(k, g);
+      const double pv = fma(beta, po[i], zz[i]);
+      ut[q.el * tile + q.pc] = pv;
+      pnew[base + k] = pv;
+    }
+  }
+  __syncthreads();                             // the neighbour bases
+  // face halos, recomputed from the neighbours' z and p_old: item = (element, face cell)
+  const int F0 = g.by * g.bz, F1 = g.bx * g.bz, F2 = g.bx * g.by, H = 2 * (F0 + F1 + F2);
+  for (int b0 = 0; b0 < ne * H; b0 += kB * kGThreads) {
+    double zv[kB], pv[kB];
+    int dst[kB];
+    bool in[kB];
+#pragma unroll
+    for (int i = 0; i < kB; ++i) {
+      const int k = b0 + kGThreads * i + (int)threadIdx.x;
+      zv[i] = pv[i] = 0.0;
+      dst[i] = -1;
+      in[i] = false;
+      if (k >= ne * H) continue;
+      const int el = k / H, h = k - el * H;
+      const int d = h < 2 * F0 ? 0 : (h < 2 * (F0 + F1) ? 1 : 2);
+      const int F = d == 0 ? F0 : (d == 1 ? F1 : F2);
+      int h1 = h - (d == 0 ? 0 : (d == 1 ? 2 * F0 : 2 * (F0 + F1)));
+      const bool plus = h1 >= F;
+      if (plus) h1 -= F;
+      const int w = d == 0 ? g.by : g.bx, vv = h1 / w, uu = h1 - vv * w;
+      int dx, dy, dz, sx, sy, sz;
+      if (d == 0) { dy = sy = uu; dz = sz = vv; dx = plus ? g.bx : -1; sx = plus ? 0 : g.bx - 1; }
+      else if (d == 1) { dx = sx = uu; dz = sz = vv; dy = plus ? g.by : -1; sy = plus ? 0 : g.by - 1; }
+      else { dx = sx = uu; dy = sy = vv; dz = plus ? g.bz : -1; sz = plus ? 0 : g.bz - 1; }
+      dst[i] = el * tile + wpad(g, dx, dy, dz);
+      const int64_t b = nb[el * 6 + 2 * d + (plus ? 1 : 0)];
+      if (b >= 0) {
+        const int64_t src = b + sx + g.bx * (sy + g.by * sz);
+        zv[i] = __ldg(z + src);
+        pv[i] = __ldg(pold + src);
+        in[i] = true;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kB; ++i)
+      if (dst[i] >= 0) ut[dst[i]] = in[i] ? fma(beta, pv[i], zv[i]) : 0.0;
+  }
+  __syncthreads();
+  const int sy = g.bx + 2, sz = (g.bx + 2) * (g.by + 2);
+  double acc = 0.0;
+  constexpr int kQ = 2;
+  for (int b0 = 0; b0 < cells; b0 += kQ * kGThreads) {
+    double t0[kQ], t1[kQ], t2[kQ], dg[kQ], mx[kQ], my[kQ], mz[kQ];
+    GCell q[kQ];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+      const int k = b0 + kGThreads * i + (int)threadIdx.x;
+      if (k >= cells) continue;
+      q[i] = grp_cell(k, g);
+      t0[i] = __ldg(T + base + k);
+      t1[i] = __ldg(T + n + base + k);
+      t2[i] = __ldg(T + 2 * n + base + k);
+      dg[i] = __ldg(Dg + base + k);
+      mx[i] = grp_tminus(T, 0, base, nb, q[i], g);
+      my[i] = grp_tminus(T + n, 1, base, nb, q[i], g);
+      mz[i] = grp_tminus(T + 2 * n, 2, base, nb, q[i], g);
+    }
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+      const int k = b0 + kGThreads * i + (int)threadIdx.x;
+      if (k >= cells) continue;
+      const double* up = ut + q[i].el * tile + q[i].pc;
+      const double pc = up[0];
+      // (A p)_c = D_c p_c - sum_f T_f p_nb: one multiply and six FMAs in FP64
+      double a = dg[i] * pc;
+      a = fma(-t0[i], up[1], a);
+      a = fma(-mx[i], up[-1], a);
+      a = fma(-t1[i], up[sy], a);
+      a = fma(-my[i], up[-sy], a);
+      a = fma(-t2[i], up[sz], a);
+      a = fma(-mz[i], up[-sz], a);
+      qo[base + k] = a;
+      acc = fma(a, pc, acc);
+    }
+  }
+  double v[1] = {acc};
+  grid_reduce_r<1>(v, red, bi, [=] __device__(double* t) {
+    sc->pq = t[0];
+    if (!(t[0] > 0.0) || !isfinite(t[0])) { sc->done = 2; sc->alpha = 0.0; }
+    else sc->alpha = sc->rz / t[0];
+  });
+}
+template <typename G>
+__host__ __device__ inline size_t grp_tile_bytes(const G& g, size_t vsize, bool residual) {
+  const Grp q = make_grp(g);
+  return (size_t)6 * q.E * sizeof(int64_t) + ((size_t)q.E * r4(g.P) + (residual ? q.E * g.nb : 0)) * vsize;
+}
+
 // ------------------------------------------------------------------ host side
 template <typename V, typename BT>
 struct FineOps {
@@ -1365,18 +2084,72 @@ static inline unsigned fine_wgrid(const msmg_ctx* c, int W = kWarpsPerCta) {
   return (unsigned)((c->fine.m + W - 1) / W * c->sb.R);
 }
 
+// a warp per element is compiled for every shape but FP32 4^3 elements, which always take groups
+template <typename V, typename G>
+constexpr bool kHasWarp = !(std::is_same<V, float>::value && std::is_same<G, GeoC<4, 4, 4>>::value);
+// Groups of elements: where a warp has a lane for every x-line of a z-plane, except 8^3
+// elements, and in FP64 except grids of few elements (a sweeping warp's FP64 chains take
+// twice as long as a warp per element's, which shows where all elements run at once:
+// 512 elements of 4^3, a solve 1.13 against 1.39 ms).
+template <typename V, typename G>
+static bool use_groups(const msmg_ctx* c, const G& g) {
+  return !IsCube8<G>::value && g.by <= 32 && (sizeof(V) == 4 || c->fine.m >= 152 * 16);
+}
+template <typename G>
+static unsigned grp_grid(const msmg_ctx* c, const G& g) {
+  const int E = make_grp(g).E;
+  return (unsigned)((c->fine.m + E - 1) / E * c->sb.R);
+}
+// cells per thread of k_post_grp's register arrays (5: 80-cell elements, 64 registers and
+// 56 us on 60 x 220 x 85 cells, where 8 take 96 and 75 us)
+template <bool FUSE, typename G, typename F>
+static void with_kc(const G& g, F&& fn) {
+  const int need = (make_grp(g).E * g.nb + kGThreads - 1) / kGThreads;
+  if constexpr (IsGeoC<G>::value) {
+    constexpr G gc{};
+    constexpr int k = (make_grp(gc).E * G::nb + kGThreads - 1) / kGThreads;
+    fn(std::integral_constant<int, k>{});
+  } else {
+    if constexpr (!FUSE)
+      if (need <= 5) return fn(std::integral_constant<int, 5>{});
+    if (need <= 8) fn(std::integral_constant<int, 8>{});
+    else fn(std::integral_constant<int, kGCells>{});
+  }
+}
+
 template <typename V, typename BT, typename G>
 static void pre_t(msmg_ctx* c, const FineOps<V, BT>& o, int update, PcgScalars* sc, cudaStream_t s, const G& g) {
   SolveBuffers& B = c->sb;
-  constexpr int W = stage_elems<kStagePre, V, G>();
-  k_pre<V, G><<<fine_wgrid(c, W), W * elem_threads<kStagePre, G, V>(), wsmem<kStagePre, V>(g), s>>>(
-      B.x, B.r, B.pcur, B.q, o.T, o.invd, (V*)B.rv, (V*)B.vu[1], c->n, g, c->fine.m, c->fine.nbr, update, c->red, sc,
-      c->flags + 6, B.R);
+  if constexpr (!IsCube8<G>::value) {
+    if (use_groups<V>(c, g)) {
+      k_pre_grp<V, G><<<grp_grid(c, g), kGThreads, grp_pre_floats(g) * sizeof(V), s>>>(
+          B.x, B.r, B.pcur, B.q, o.T, o.invd, (V*)B.rv, (V*)B.vu[1], c->n, g, c->fine.m, update, c->red, sc,
+          c->flags + 6, B.R);
+      return;
+    }
+  }
+  if constexpr (kHasWarp<V, G>) {
+    constexpr int W = stage_elems<kStagePre, V, G>();
+    k_pre<V, G><<<fine_wgrid(c, W), W * elem_threads<kStagePre, G, V>(), wsmem<kStagePre, V>(g), s>>>(
+        B.x, B.r, B.pcur, B.q, o.T, o.invd, (V*)B.rv, (V*)B.vu[1], c->n, g, c->fine.m, c->fine.nbr, update, c->red, sc,
+        c->flags + 6, B.R);
+  }
 }
 
 template <typename V, typename BT, typename G>
 static void restrict_t(msmg_ctx* c, const FineOps<V, BT>& o, PcgScalars* sc, cudaStream_t s, const G& g) {
   SolveBuffers& B = c->sb;
+  // groups only from 16 elements per SM (60 x 220 x 85: 61 -> 47 us; 288 elements of 4 x 4 x 5,
+  // three right-hand sides: 14 -> 16), and not on 4^3, whose warps have two full cells a lane
+  // (72 x 48 x 104: 12.2 against 14.2 us)
+  if constexpr (!IsGeoC<G>::value) {
+    if (use_groups<V>(c, g) && c->fine.m >= 152 * 16) {
+      k_restrict_grp<V, BT, G><<<grp_grid(c, g), kGThreads, grp_tile_bytes(g, sizeof(V), true), s>>>(
+          (const V*)B.rv, (const V*)B.vu[1], o.T, o.Wd, o.Phi, c->fine.L, (double*)B.vf[2], c->lev[2].n, c->n, g,
+          c->fine.m, c->fine.nbr, sc, B.R);
+      return;
+    }
+  }
   constexpr int W = stage_elems<restrict_layout<V>(), V>();
   k_restrict<V, BT, G><<<fine_wgrid(c, W), W * 32, wsmem<restrict_layout<V>(), V>(g), s>>>(
       (const V*)B.rv, (const V*)B.vu[1], o.T, o.Wd, o.Phi, c->fine.L, (double*)B.vf[2], c->lev[2].n, c->n, g, c->fine.m,
@@ -1387,16 +2160,31 @@ template <typename V, typename BT, typename G>
 static void post_t(msmg_ctx* c, const FineOps<V, BT>& o, const V* ec, const double* qv, PcgScalars* sc,
                    cudaStream_t s, const G& g, bool fuse) {
   SolveBuffers& B = c->sb;
-  constexpr int W = stage_elems<kStageFull, V, G>();
-  constexpr int NT = elem_threads<kStageFull, G, V>();
-  if (fuse)
-    k_post<V, BT, G, true><<<fine_wgrid(c, W), W * NT, wsmem<kStageFull, V>(g), s>>>(
-        (const V*)B.rv, B.r, (const V*)B.vu[1], o.T, o.Wd, o.invd, o.Phi, ec, c->fine.L, c->lev[2].n, B.z, qv, c->n, g,
-        c->fine.m, c->fine.nbr, c->red, sc, c->flags + 6, B.R, B.R > 1 ? c->pf_post[1] : 0);
-  else
-    k_post<V, BT, G, false><<<fine_wgrid(c, W), W * NT, wsmem<kStageFull, V>(g), s>>>(
-        (const V*)B.rv, B.r, (const V*)B.vu[1], o.T, o.Wd, o.invd, o.Phi, ec, c->fine.L, c->lev[2].n, B.z, qv, c->n, g,
-        c->fine.m, c->fine.nbr, c->red, sc, c->flags + 6, B.R, B.R > 1 ? c->pf_post[0] : 0);
+  if constexpr (!IsCube8<G>::value) {
+    if (use_groups<V>(c, g)) {
+      auto run = [&](auto k, int pf) {
+        k<<<grp_grid(c, g), kGThreads, grp_post_floats(g) * sizeof(V), s>>>(
+            (const V*)B.rv, B.r, (const V*)B.vu[1], o.T, o.Wd, o.invd, o.Phi, ec, c->fine.L, c->lev[2].n, B.z, qv,
+            c->n, g, c->fine.m, c->fine.nbr, c->red, sc, c->flags + 6, B.R, pf);
+      };
+      const int pf = B.R > 1 ? c->pf_post[fuse ? 1 : 0] : 0;
+      if (fuse) with_kc<true>(g, [&](auto kc) { run(k_post_grp<V, G, true, decltype(kc)::value>, pf); });
+      else with_kc<false>(g, [&](auto kc) { run(k_post_grp<V, G, false, decltype(kc)::value>, pf); });
+      return;
+    }
+  }
+  if constexpr (kHasWarp<V, G>) {
+    constexpr int W = stage_elems<kStageFull, V, G>();
+    constexpr int NT = elem_threads<kStageFull, G, V>();
+    if (fuse)
+      k_post<V, BT, G, true><<<fine_wgrid(c, W), W * NT, wsmem<kStageFull, V>(g), s>>>(
+          (const V*)B.rv, B.r, (const V*)B.vu[1], o.T, o.Wd, o.invd, o.Phi, ec, c->fine.L, c->lev[2].n, B.z, qv, c->n, g,
+          c->fine.m, c->fine.nbr, c->red, sc, c->flags + 6, B.R, B.R > 1 ? c->pf_post[1] : 0);
+    else
+      k_post<V, BT, G, false><<<fine_wgrid(c, W), W * NT, wsmem<kStageFull, V>(g), s>>>(
+          (const V*)B.rv, B.r, (const V*)B.vu[1], o.T, o.Wd, o.invd, o.Phi, ec, c->fine.L, c->lev[2].n, B.z, qv, c->n, g,
+          c->fine.m, c->fine.nbr, c->red, sc, c->flags + 6, B.R, B.R > 1 ? c->pf_post[0] : 0);
+  }
 }
 
 template <typename V, typename BT, typename G>
@@ -1417,6 +2205,13 @@ static void prolong_t(msmg_ctx* c, const FineOps<V, BT>& o, const V* ec, PcgScal
 template <typename G>
 static void pmatvec_t(msmg_ctx* c, PcgScalars* sc, cudaStream_t s, const G& g) {
   SolveBuffers& B = c->sb;
+  if constexpr (!IsCube8<G>::value) {
+    if (use_groups<double>(c, g)) {
+      k_pmatvec_grp<G><<<grp_grid(c, g), kGThreads, grp_tile_bytes(g, sizeof(double), false), s>>>(
+          B.z, B.pcur, B.pnext, B.q, c->fine.T, c->fine.D, c->n, g, c->fine.m, c->fine.nbr, c->red, sc, B.R);
+      return;
+    }
+  }
   k_pmatvec<G><<<fine_wgrid(c, kPmWarps), kPmWarps * 32, wsmem_p(g), s>>>(B.z, B.pcur, B.pnext, B.q, c->fine.T, c->fine.D,
                                                                       c->n, g, c->fine.m, c->fine.nbr, c->red, sc, B.R);
 }
@@ -1437,23 +2232,37 @@ static int resident_ctas(const void* k, int threads, size_t smem) {
 
 template <typename V, typename BT, typename G>
 static void prepare_t(msmg_ctx* c, const G& g) {
-  const int smv = (int)wsmem<kStageFull, V>(g), smd = (int)wsmem_p(g);
-  cudaFuncSetAttribute(k_pre<V, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsmem<kStagePre, V>(g));
-  cudaFuncSetAttribute(k_restrict<V, BT, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)wsmem<restrict_layout<V>(), V>(g));
-  cudaFuncSetAttribute(k_restrict<V, BT, G>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                       cudaSharedmemCarveoutMaxShared);
-  cudaFuncSetAttribute(k_post<V, BT, G, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smv);
-  cudaFuncSetAttribute(k_post<V, BT, G, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smv);
-  cudaFuncSetAttribute(k_post<V, BT, G, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                       cudaSharedmemCarveoutMaxShared);
-  cudaFuncSetAttribute(k_post<V, BT, G, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                       cudaSharedmemCarveoutMaxShared);
-  cudaFuncSetAttribute(k_pmatvec<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
-  cudaFuncSetAttribute(k_pmatvec<G>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  constexpr int NT = elem_threads<kStageFull, G, V>();
-  c->pf_post[0] = resident_ctas((const void*)k_post<V, BT, G, false>, stage_elems<kStageFull, V, G>() * NT, smv);
-  c->pf_post[1] = resident_ctas((const void*)k_post<V, BT, G, true>, stage_elems<kStageFull, V, G>() * NT, smv);
+  auto smem = [](auto k, size_t bytes, bool carve) {
+    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (carve) cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  };
+  if constexpr (!IsCube8<G>::value) {
+    if (use_groups<double>(c, g)) smem(k_pmatvec_grp<G>, grp_tile_bytes(g, sizeof(double), false), true);
+    if (use_groups<V>(c, g)) {
+      smem(k_pre_grp<V, G>, grp_pre_floats(g) * sizeof(V), true);
+      if constexpr (!IsGeoC<G>::value) smem(k_restrict_grp<V, BT, G>, grp_tile_bytes(g, sizeof(V), true), true);
+      const size_t so = grp_post_floats(g) * sizeof(V);
+      auto post = [&](auto k, int i) {
+        smem(k, so, true);
+        c->pf_post[i] = resident_ctas((const void*)k, kGThreads, so);
+      };
+      with_kc<false>(g, [&](auto kc) { post(k_post_grp<V, G, false, decltype(kc)::value>, 0); });
+      with_kc<true>(g, [&](auto kc) { post(k_post_grp<V, G, true, decltype(kc)::value>, 1); });
+    }
+  }
+  smem(k_pmatvec<G>, wsmem_p(g), true);
+  smem(k_restrict<V, BT, G>, wsmem<restrict_layout<V>(), V>(g), true);
+  if constexpr (kHasWarp<V, G>) {
+    if (!use_groups<V>(c, g)) {
+      const size_t smv = wsmem<kStageFull, V>(g);
+      smem(k_pre<V, G>, wsmem<kStagePre, V>(g), false);
+      smem(k_post<V, BT, G, true>, smv, true);
+      smem(k_post<V, BT, G, false>, smv, true);
+      constexpr int NT = elem_threads<kStageFull, G, V>();
+      c->pf_post[0] = resident_ctas((const void*)k_post<V, BT, G, false>, stage_elems<kStageFull, V, G>() * NT, smv);
+      c->pf_post[1] = resident_ctas((const void*)k_post<V, BT, G, true>, stage_elems<kStageFull, V, G>() * NT, smv);
+    }
+  }
 }
 
 void prepare_fine_kernels(msmg_ctx* c) {
