@@ -81,7 +81,7 @@ __device__ __forceinline__ S ld_vec(const S* p) {
 // one thread in turn (fused forms) give the same bits.
 template <int LT, typename S, bool NC = true>
 __device__ __forceinline__ S coarse_residual_part(const CoarseLevel& lv, const LevelData<S>& D, int64_t P, int t,
-                                                  int s, const S* __restrict__ f, const S* __restrict__ u) {
+                                                  int s, const S* f, const S* u) {
   const int L = LT ? LT : lv.L;
   const int64_t a = P * lv.nchild + t / L;
   const int k = t % L;
@@ -127,12 +127,89 @@ __device__ __forceinline__ S coarse_residual_part(const CoarseLevel& lv, const L
 
 template <int LT, typename S, bool NC = true>
 __device__ __forceinline__ S coarse_residual_row(const CoarseLevel& lv, const LevelData<S>& D, int64_t P, int t,
-                                                 const S* __restrict__ f, const S* __restrict__ u) {
+                                                 const S* f, const S* u) {
   const S p0 = coarse_residual_part<LT, S, NC>(lv, D, P, t, 0, f, u);
   const S p1 = coarse_residual_part<LT, S, NC>(lv, D, P, t, 1, f, u);
   const S p2 = coarse_residual_part<LT, S, NC>(lv, D, P, t, 2, f, u);
   const S p3 = coarse_residual_part<LT, S, NC>(lv, D, P, t, 3, f, u);
   return (p0 + p1) + (p2 + p3);
+}
+
+// The four partials of a row by four threads of a warp (per-level kernels, QUAD): thread s
+// takes partial s, the same sums as coarse_residual_part, but with one code path: every
+// thread subtracts a first block (own, or +d neighbour) and a second one (none, or -d).
+// As divergent branches the two kinds of partials ran one after the other, with their
+// loads.  load() reads what set-up wrote (the row's neighbours and coefficients) and may
+// run before the kernel waits for the previous launch; sum() reads f and u.
+template <int LT, typename S>
+struct ResidualPart {
+  const S *a1, *a2;
+  int64_t own;                          // f and u offset of the row's element
+  int b1, b2;                           // elements of the two blocks, -1: none
+  int k, L;
+  bool first;                           // partial 0: starts from f
+  S c1[LT ? LT : 1], c2[LT ? LT : 1];
+  __device__ __forceinline__ void load(const CoarseLevel& lv, const LevelData<S>& D, int64_t P, int t, int s, bool on) {
+    L = LT ? LT : lv.L;
+    const int64_t a = P * lv.nchild + t / L;
+    const int L2 = L * L, d = s - 1;
+    k = t % L;
+    own = a * L;
+    first = s == 0;
+    b1 = b2 = -1;
+    a1 = a2 = nullptr;
+    if (!on) return;
+    b1 = first ? (int)a : __ldg(lv.nbr + a * 6 + 2 * d + 1);
+    b2 = first ? -1 : __ldg(lv.nbr + a * 6 + 2 * d);
+    a1 = first ? D.Ad + a * L2 + (size_t)k * L : D.Ao + ((size_t)a * 3 + d) * L2 + (size_t)k * L;
+    if (b2 >= 0) a2 = D.Ao + ((size_t)b2 * 3 + d) * L2 + k;
+    if (LT) {
+#pragma unroll
+      for (int mm = 0; mm < LT; ++mm) {
+        c1[mm] = b1 >= 0 ? __ldg(a1 + mm) : (S)0;
+        c2[mm] = b2 >= 0 ? __ldg(a2 + (size_t)mm * LT) : (S)0;
+      }
+    }
+  }
+  __device__ __forceinline__ S sum(const S* f, const S* u) const {
+    S acc = first ? f[own + k] : (S)0;
+    if (LT) {
+      S u1[LT ? LT : 1], u2[LT ? LT : 1];
+#pragma unroll
+      for (int mm = 0; mm < LT; ++mm) {
+        u1[mm] = b1 >= 0 ? u[(int64_t)b1 * LT + mm] : (S)0;
+        u2[mm] = b2 >= 0 ? u[(int64_t)b2 * LT + mm] : (S)0;
+      }
+      if (b1 >= 0) {
+#pragma unroll
+        for (int mm = 0; mm < LT; ++mm) acc -= c1[mm] * u1[mm];
+      }
+      if (b2 >= 0) {
+#pragma unroll
+        for (int mm = 0; mm < LT; ++mm) acc -= c2[mm] * u2[mm];
+      }
+    } else {
+      if (b1 >= 0)
+        for (int mm = 0; mm < L; ++mm) acc -= __ldg(a1 + mm) * u[(int64_t)b1 * L + mm];
+      if (b2 >= 0)
+        for (int mm = 0; mm < L; ++mm) acc -= __ldg(a2 + (size_t)mm * L) * u[(int64_t)b2 * L + mm];
+    }
+    return acc;
+  }
+};
+
+// The warp sums of four values, by exchanging halves: 6 additions instead of 20, the pairs
+// of warp_sum_t at every step, so the same bits.  Returned: in lanes 0, 16, 8, 24 the sums
+// of v0, v1, v2, v3.
+template <typename S>
+__device__ __forceinline__ S warp_sum4(S v0, S v1, S v2, S v3) {
+  const bool h = threadIdx.x & 16, q = threadIdx.x & 8;
+  S a = (h ? v1 : v0) + __shfl_xor_sync(0xffffffffu, h ? v0 : v1, 16);
+  const S b = (h ? v3 : v2) + __shfl_xor_sync(0xffffffffu, h ? v2 : v3, 16);
+  a = (q ? b : a) + __shfl_xor_sync(0xffffffffu, q ? a : b, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
 }
 
 // (q0 + q1) + (q2 + q3) of the four lanes 4t .. 4t+3 of a warp, in every one of them
@@ -181,18 +258,25 @@ __host__ __device__ inline unsigned coarse_threads4_d(int nP, int Ln) {
   return (unsigned)((t + 31) / 32 * 32);
 }
 
+// The per-level kernels follow one another at once (launch_next: a launch may start while
+// the one before it runs): each loads what set-up wrote -- smoother inverse, basis,
+// coefficients -- then waits for the launch before it (prev_wait) before it reads f, u or
+// the solve's state, and lets the next one start (next_start).  Every CTA waits before it
+// exits, so a launch has ended only when all before it have.  What an earlier launch wrote
+// is read with plain loads, not through the read-only path, which is for data that does
+// not change while a kernel runs.  Latency binds these kernels (2 to 20 us each): with the
+// one-path residuals and the four sums at a time below, 128^3 coarse levels 70 -> 47 us
+// launched singly, a whole iteration in the graph 232 -> 225; 32^3 75 -> 72;
+// 60 x 220 x 85 278 -> 271.  Letting the fine restriction start the first coarse launch
+// as well cost 72 x 48 x 104 8 us, so that one waits for its end.
+
 // Row layouts of the per-level kernels, the same bits either way: QUAD, four
 // threads per row (a level with few parents: shorter dependent chains, more
 // warps); otherwise thread t takes row t and forms the four partials in turn.
 // Pre-smoothing from zero on level l: u_P = Minv_P f_P.
 template <typename S, bool QUAD>
-__global__ void k_coarse_smooth_first(CoarseLevel lv, LevelData<S> D, const S* __restrict__ f, S* __restrict__ u,
-                                      const PcgScalars* sc, int R) {
+__global__ void k_coarse_smooth_first(CoarseLevel lv, LevelData<S> D, const S* f, S* u, const PcgScalars* sc, int R) {
   const BatchIdx bi = batch_idx(R);
-  if (sc) sc += bi.r;
-  if (sc && sc->done) return;
-  f += (int64_t)bi.r * lv.n;
-  u += (int64_t)bi.r * lv.n;
   extern __shared__ __align__(16) unsigned char smraw[];
   S* sm = reinterpret_cast<S*>(smraw);
   const int64_t P = bi.blk;
@@ -200,8 +284,13 @@ __global__ void k_coarse_smooth_first(CoarseLevel lv, LevelData<S> D, const S* _
   S* Mi = sm;                      // [nP][nP]
   S* fs = sm + (size_t)nP * nP;
   cta_cp(Mi, D.Minv + (size_t)P * nP * nP, nP * nP);
+  prev_wait();
+  next_start();
+  if (sc && sc[bi.r].done) { cp_wait(); return; }
+  f += (int64_t)bi.r * lv.n;
+  u += (int64_t)bi.r * lv.n;
   const int t = threadIdx.x;
-  if (t < nP) fs[t] = __ldg(f + P * nP + t);
+  if (t < nP) fs[t] = f[P * nP + t];
   cp_wait();
   __syncthreads();
   if constexpr (QUAD) {
@@ -216,16 +305,11 @@ __global__ void k_coarse_smooth_first(CoarseLevel lv, LevelData<S> D, const S* _
 
 // Residual and restriction to level l+1: fn[P][j] = sum_i Psi[P][j][i] (f - A_l u)_i.
 // The residual rows by four threads each; the sums over the rows in the warps of
-// the row-per-thread layout (the order of the fused forms).
+// the row-per-thread layout (the order of the fused forms), four at a time.
 template <int LT, typename S, bool QUAD>
-__global__ void k_coarse_resid_restrict(CoarseLevel lv, LevelData<S> D, const S* __restrict__ f,
-                                        const S* __restrict__ u, S* __restrict__ fn, const PcgScalars* sc, int R) {
+__global__ void k_coarse_resid_restrict(CoarseLevel lv, LevelData<S> D, const S* f, const S* u, S* fn,
+                                        const PcgScalars* sc, int R) {
   const BatchIdx bi = batch_idx(R);
-  if (sc) sc += bi.r;
-  if (sc && sc->done) return;
-  f += (int64_t)bi.r * lv.n;
-  u += (int64_t)bi.r * lv.n;
-  fn += (int64_t)bi.r * lv.mP * lv.Lnext;
   extern __shared__ __align__(16) unsigned char smraw[];
   S* sm = reinterpret_cast<S*>(smraw);
   const int64_t P = bi.blk;
@@ -235,24 +319,35 @@ __global__ void k_coarse_resid_restrict(CoarseLevel lv, LevelData<S> D, const S*
   S* red = sm + (size_t)Ln * nP;         // [Ln][nw]
   S* rs = red + (size_t)Ln * nw;         // [nP] residual rows
   cta_cp(ps, D.Psi + (size_t)P * Ln * nP, Ln * nP);
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, row = t >> 2;
+  ResidualPart<LT, S> rp;
+  if constexpr (QUAD) rp.load(lv, D, P, row, t & 3, row < nP);
+  prev_wait();
+  next_start();
+  if (sc && sc[bi.r].done) { cp_wait(); return; }
+  f += (int64_t)bi.r * lv.n;
+  u += (int64_t)bi.r * lv.n;
+  fn += (int64_t)bi.r * lv.mP * lv.Lnext;
   if constexpr (QUAD) {
-    const int row = t >> 2, sub = t & 3;
-    S q = row < nP ? coarse_residual_part<LT>(lv, D, P, row, sub, f, u) : (S)0;
+    S q = row < nP ? rp.sum(f, u) : (S)0;
     q = quad_combine(q);
-    if (row < nP && sub == 0) rs[row] = q;
+    if (row < nP && (t & 3) == 0) rs[row] = q;
   } else {
-    if (t < nP) rs[t] = coarse_residual_row<LT>(lv, D, P, t, f, u);
+    if (t < nP) rs[t] = coarse_residual_row<LT, S, false>(lv, D, P, t, f, u);
   }
   cp_wait();
   __syncthreads();
   if (t < nw * 32) {
     const int lane = t & 31, w = t >> 5;
-    const S rt = t < nP ? rs[t] : (S)0;
-    for (int j = 0; j < Ln; ++j) {
-      S v = t < nP ? ps[(size_t)j * nP + t] * rt : (S)0;
-      v = warp_sum_t(v);
-      if (lane == 0) red[j * nw + w] = v;
+    const bool on = t < nP;
+    const S rt = on ? rs[t] : (S)0;
+    for (int j = 0; j < Ln; j += 4) {
+      S v[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = on && j + i < Ln ? ps[(size_t)(j + i) * nP + t] * rt : (S)0;
+      const S a = warp_sum4(v[0], v[1], v[2], v[3]);
+      const int i = (lane >> 4) + 2 * (lane >> 3 & 1);
+      if ((lane & 7) == 0 && j + i < Ln) red[(j + i) * nw + w] = a;
     }
   }
   __syncthreads();
@@ -265,37 +360,37 @@ __global__ void k_coarse_resid_restrict(CoarseLevel lv, LevelData<S> D, const S*
 
 // Prolongation: u_P += Psi_P^T e_P.
 template <typename S>
-__global__ void k_coarse_prolong(CoarseLevel lv, LevelData<S> D, S* __restrict__ u, const S* __restrict__ e,
-                                 const PcgScalars* sc, int R) {
+__global__ void k_coarse_prolong(CoarseLevel lv, LevelData<S> D, S* u, const S* e, const PcgScalars* sc, int R) {
   const BatchIdx bi = batch_idx(R);
-  if (sc) sc += bi.r;
-  if (sc && sc->done) return;
-  u += (int64_t)bi.r * lv.n;
-  e += (int64_t)bi.r * lv.mP * lv.Lnext;
   const int64_t P = bi.blk;
-  const int t = threadIdx.x;
-  if (t >= lv.nP) return;
-  const S* ps = D.Psi + (size_t)P * lv.Lnext * lv.nP;
+  const int t = threadIdx.x, Ln = lv.Lnext;
+  const bool on = t < lv.nP;
+  const S* ps = D.Psi + (size_t)P * Ln * lv.nP;
+  constexpr int kPre = 8;                // basis values held in registers across the wait
+  S p[kPre];
+#pragma unroll
+  for (int j = 0; j < kPre; ++j) p[j] = on && j < Ln ? __ldg(ps + (size_t)j * lv.nP + t) : (S)0;
+  prev_wait();
+  next_start();
+  if (sc && sc[bi.r].done) return;
+  if (!on) return;
+  u += (int64_t)bi.r * lv.n;
+  e += (int64_t)bi.r * lv.mP * Ln;
   S acc = 0;
+#pragma unroll
+  for (int j = 0; j < kPre; ++j)
+    if (j < Ln) acc = fma(p[j], e[P * Ln + j], acc);
 #pragma unroll 4
-  for (int j = 0; j < lv.Lnext; ++j) acc = fma(__ldg(ps + (size_t)j * lv.nP + t), __ldg(e + P * lv.Lnext + j), acc);
+  for (int j = kPre; j < Ln; ++j) acc = fma(__ldg(ps + (size_t)j * lv.nP + t), e[P * Ln + j], acc);
   u[P * lv.nP + t] += acc;
 }
 
 // Post-smoothing: out = u + Minv (f - A_l u)   (out must not alias u); the residual
 // rows and the smoother GEMV by four threads per row.
 template <int LT, typename S, bool QUAD>
-__global__ void k_coarse_resid_smooth(CoarseLevel lv, LevelData<S> D, const S* __restrict__ f,
-                                      const S* __restrict__ u, S* __restrict__ out, float* __restrict__ out32,
+__global__ void k_coarse_resid_smooth(CoarseLevel lv, LevelData<S> D, const S* f, const S* u, S* out, float* out32,
                                       const PcgScalars* sc, int R) {
   const BatchIdx bi = batch_idx(R);
-  if (sc) sc += bi.r;
-  if (sc && sc->done) return;
-  {
-    const int64_t off = (int64_t)bi.r * lv.n;
-    f += off; u += off; out += off;
-    if (out32) out32 += off;
-  }
   extern __shared__ __align__(16) unsigned char smraw[];
   S* sm = reinterpret_cast<S*>(smraw);
   const int64_t P = bi.blk;
@@ -304,9 +399,19 @@ __global__ void k_coarse_resid_smooth(CoarseLevel lv, LevelData<S> D, const S* _
   S* rs = sm + (size_t)nP * nP;
   cta_cp(Mi, D.Minv + (size_t)P * nP * nP, nP * nP);
   const int t = threadIdx.x;
+  ResidualPart<LT, S> rp;
+  if constexpr (QUAD) rp.load(lv, D, P, t >> 2, t & 3, (t >> 2) < nP);
+  prev_wait();
+  next_start();
+  if (sc && sc[bi.r].done) { cp_wait(); return; }
+  {
+    const int64_t off = (int64_t)bi.r * lv.n;
+    f += off; u += off; out += off;
+    if (out32) out32 += off;
+  }
   if constexpr (QUAD) {
     const int row = t >> 2, sub = t & 3;
-    S q = row < nP ? coarse_residual_part<LT>(lv, D, P, row, sub, f, u) : (S)0;
+    S q = row < nP ? rp.sum(f, u) : (S)0;
     q = quad_combine(q);
     if (row < nP && sub == 0) rs[row] = q;
     cp_wait();
@@ -319,7 +424,7 @@ __global__ void k_coarse_resid_smooth(CoarseLevel lv, LevelData<S> D, const S* _
       if (out32) out32[P * nP + row] = (float)v;
     }
   } else {
-    if (t < nP) rs[t] = coarse_residual_row<LT>(lv, D, P, t, f, u);
+    if (t < nP) rs[t] = coarse_residual_row<LT, S, false>(lv, D, P, t, f, u);
     cp_wait();
     __syncthreads();
     if (t < nP) {
@@ -360,10 +465,11 @@ __device__ __forceinline__ double coarsest_row(const double* __restrict__ A, con
 }
 
 template <typename S>
-__global__ void k_dense_gemv(const double* __restrict__ A, const S* __restrict__ x, S* __restrict__ y,
-                             float* __restrict__ y32, int64_t n, int64_t nk, const int* __restrict__ cmap,
-                             const int* __restrict__ cinv, const PcgScalars* sc, int R) {
+__global__ void k_dense_gemv(const double* __restrict__ A, const S* x, S* y, float* y32, int64_t n, int64_t nk,
+                             const int* __restrict__ cmap, const int* __restrict__ cinv, const PcgScalars* sc, int R) {
   const BatchIdx bi = batch_idx(R);
+  prev_wait();
+  next_start();
   if (sc) sc += bi.r;
   if (sc && sc->done) return;
   x += (int64_t)bi.r * n;
@@ -1129,6 +1235,23 @@ int coarse_forms(const msmg_ctx* c) {
 }
 
 
+// Launch that may start while the launch before it runs; the kernel waits for that one
+// itself (prev_wait).  After anything but a kernel it starts when that has ended.
+template <typename... P, typename... A>
+static void launch_next(void (*k)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, P(args)...);
+}
+
 // Level-l part of the V-cycle (l >= 2): on entry vf[l] holds the right side;
 // returns the device pointer holding the level-l correction.
 template <typename S>
@@ -1153,8 +1276,8 @@ static const S* coarse_cycle_t(msmg_ctx* c, int l, PcgScalars* sc, cudaStream_t 
   }
   if (l == c->nL) {
     const unsigned grid = (unsigned)((lv.n * 32 + 255) / 256 * R);
-    k_dense_gemv<S><<<grid, 256, 0, s>>>(lv.pinv, f, u, l == 2 ? c->sb.ec32 : nullptr, lv.n, lv.nk, lv.cmap,
-                                         lv.cinv, sc, R);
+    launch_next(k_dense_gemv<S>, grid, 256, 0, s, lv.pinv, f, u, l == 2 ? c->sb.ec32 : nullptr, lv.n, lv.nk, lv.cmap,
+                lv.cinv, sc, R);
     return u;
   }
   const LevelData<S> D = level_data<S>(lv);
@@ -1163,22 +1286,22 @@ static const S* coarse_cycle_t(msmg_ctx* c, int l, PcgScalars* sc, cudaStream_t 
   // four threads per row when the level's CTAs leave the GPU short of warps
   const bool quad = grid < (unsigned)(152 * 8);
   const unsigned thr = coarse_threads(lv), thrs = quad ? coarse_threads4(lv) : thr;
-  if (quad) k_coarse_smooth_first<S, true><<<grid, thrs, smem_smooth<S>(lv), s>>>(lv, D, f, u, sc, R);
-  else k_coarse_smooth_first<S, false><<<grid, thrs, smem_smooth<S>(lv), s>>>(lv, D, f, u, sc, R);
+  if (quad) launch_next(k_coarse_smooth_first<S, true>, grid, thrs, smem_smooth<S>(lv), s, lv, D, f, u, sc, R);
+  else launch_next(k_coarse_smooth_first<S, false>, grid, thrs, smem_smooth<S>(lv), s, lv, D, f, u, sc, R);
   with_L(lv.L, [&](auto LC) {
     constexpr int LT = decltype(LC)::value;
     if (quad)
-      k_coarse_resid_restrict<LT, S, true><<<grid, thrs, smem_restrict<S>(lv), s>>>(lv, D, f, u, fn, sc, R);
+      launch_next(k_coarse_resid_restrict<LT, S, true>, grid, thrs, smem_restrict<S>(lv), s, lv, D, f, u, fn, sc, R);
     else
-      k_coarse_resid_restrict<LT, S, false><<<grid, thrs, smem_restrict<S>(lv), s>>>(lv, D, f, u, fn, sc, R);
+      launch_next(k_coarse_resid_restrict<LT, S, false>, grid, thrs, smem_restrict<S>(lv), s, lv, D, f, u, fn, sc, R);
   });
   const S* e = coarse_cycle_t<S>(c, l + 1, sc, s);
-  k_coarse_prolong<S><<<grid, thr, 0, s>>>(lv, D, u, e, sc, R);
+  launch_next(k_coarse_prolong<S>, grid, thr, 0, s, lv, D, u, e, sc, R);
   with_L(lv.L, [&](auto LC) {
     constexpr int LT = decltype(LC)::value;
     float* o32 = l == 2 ? c->sb.ec32 : nullptr;
-    if (quad) k_coarse_resid_smooth<LT, S, true><<<grid, thrs, smem_smooth<S>(lv), s>>>(lv, D, f, u, w, o32, sc, R);
-    else k_coarse_resid_smooth<LT, S, false><<<grid, thrs, smem_smooth<S>(lv), s>>>(lv, D, f, u, w, o32, sc, R);
+    if (quad) launch_next(k_coarse_resid_smooth<LT, S, true>, grid, thrs, smem_smooth<S>(lv), s, lv, D, f, u, w, o32, sc, R);
+    else launch_next(k_coarse_resid_smooth<LT, S, false>, grid, thrs, smem_smooth<S>(lv), s, lv, D, f, u, w, o32, sc, R);
   });
   return w;
 }

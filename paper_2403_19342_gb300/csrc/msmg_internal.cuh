@@ -263,6 +263,11 @@ __device__ __forceinline__ T warp_sum_t(T v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// Overlapping launches: prev_wait() returns when the launch before this one has ended and
+// its writes are visible (at once where there was nothing to overlap with); next_start()
+// lets the launch after this one start, which then waits for this one's end itself.
+__device__ __forceinline__ void prev_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void next_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
