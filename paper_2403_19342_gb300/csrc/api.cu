@@ -403,10 +403,11 @@ int msmg_setup(const msmg_grid* grid, const void* kappa, int kappa_components, i
   cudaEventCreate(&c->ev0);
   cudaEventCreate(&c->ev1);
   // untuned defaults: separate prolongation and a launch per coarse step, the fastest of the
-  // variants on every hierarchy they were timed on (us per iteration, best / the fused
+  // variants on every hierarchy they were timed on (us per iteration, these / the fused
   // prolongation / the cooperative coarse cycle: 32^3 FP64 76 / 78 / 91, 96^3 FP64
   // 298 / 317 / 328, 256^3 mixed 1297 / 1351 / 1366, 60x220x85 with wells 423 / 501 / 477,
-  // 96^3 with 16 right-hand sides 969 / 1013 / 996)
+  // 96^3 with 16 right-hand sides 969 / 1013 / 996; since then the launches overlap and
+  // groups of elements came: 72, 295, 1288, 271 and 966)
   c->tune_fused[0] = c->tune_fused[1] = 0;
   c->tune_tail[0] = c->tune_tail[1] = 0;
   for (int k = 0; k < 3; ++k) cudaEventCreateWithFlags(&c->poll_evs[k], cudaEventDisableTiming);
