@@ -1000,14 +1000,14 @@ static void prepare_t(msmg_ctx* c) {
   for (int l = 2; l < c->nL; ++l) {
     CoarseLevel& lv = c->lev[l];
     const int sm1 = (int)smem_smooth<S>(lv), sm2 = (int)smem_restrict<S>(lv);
-    cudaFuncSetAttribute(k_coarse_smooth_first<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1);
-    cudaFuncSetAttribute(k_coarse_smooth_first<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1);
+    smem_at_least(k_coarse_smooth_first<S, false>, sm1);
+    smem_at_least(k_coarse_smooth_first<S, true>, sm1);
     with_L(lv.L, [&](auto LC) {
       constexpr int LT = decltype(LC)::value;
-      cudaFuncSetAttribute(k_coarse_resid_smooth<LT, S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1);
-      cudaFuncSetAttribute(k_coarse_resid_smooth<LT, S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm1);
-      cudaFuncSetAttribute(k_coarse_resid_restrict<LT, S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2);
-      cudaFuncSetAttribute(k_coarse_resid_restrict<LT, S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm2);
+      smem_at_least(k_coarse_resid_smooth<LT, S, false>, sm1);
+      smem_at_least(k_coarse_resid_smooth<LT, S, true>, sm1);
+      smem_at_least(k_coarse_resid_restrict<LT, S, false>, sm2);
+      smem_at_least(k_coarse_resid_restrict<LT, S, true>, sm2);
     });
   }
 }
@@ -1043,7 +1043,7 @@ static bool tail_shape(const msmg_ctx* c, int l0, int* lt_out, size_t* sm_out) {
 
 template <int LT>
 static void cluster_prepare_lt(msmg_ctx* c) {
-  cudaFuncSetAttribute(k_coarse_tail<LT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->tail_smem);
+  smem_at_least(k_coarse_tail<LT>, c->tail_smem);
   cudaFuncSetAttribute(k_coarse_tail<LT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   for (int cs : {16, 8}) {
     cudaLaunchConfig_t cfg = {};
@@ -1075,7 +1075,7 @@ static void coop_prepare_lt(msmg_ctx* c) {
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (!coop || nsm < 1) return;
-  cudaFuncSetAttribute(k_coarse_coop<LT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->coop_smem);
+  smem_at_least(k_coarse_coop<LT>, c->coop_smem);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_coarse_coop<LT>, kTailThreads, c->coop_smem) !=
           cudaSuccess || per < 1) {
     cudaGetLastError();
@@ -1169,7 +1169,7 @@ static void inner_prepare_lt(msmg_ctx* c) {
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (!coop || nsm < 1) return;
-  cudaFuncSetAttribute(k_inner_pcg<LT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c->coop_smem);
+  smem_at_least(k_inner_pcg<LT>, c->coop_smem);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_inner_pcg<LT>, kTailThreads, c->coop_smem) !=
           cudaSuccess || per < 1) {
     cudaGetLastError();

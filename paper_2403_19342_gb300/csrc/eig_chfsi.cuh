@@ -702,7 +702,7 @@ void launch_eig_phase(msmg_ctx* c, const EigPhase& p, cudaStream_t s) {
   auto run = [&](auto kt, auto ct) {
     constexpr int KT = decltype(kt)::value, CPT = decltype(ct)::value;
     const size_t sm = chfsi_smem(f.nb, p.K, sizeof(R));
-    cudaFuncSetAttribute(k_eig_l1_chfsi<R, KT, CPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    smem_at_least(k_eig_l1_chfsi<R, KT, CPT>, sm);
     k_eig_l1_chfsi<R, KT, CPT><<<(unsigned)f.m, (unsigned)chfsi_threads(f.nb), sm, s>>>(
         f.T, f.S, c->n, f.bx, f.by, f.bz, f.m, p.L, p.K, p.max_iter, p.tol, p.guess, p.guess_vecs, p.block_out,
         p.block_out ? nullptr : f.Phi, p.block_out ? nullptr : f.lam, c->dtmp, c->flags, f.Wd);

@@ -293,7 +293,7 @@ void launch_faces(msmg_ctx* c, const void* kappa, int comps, int dtype, cudaStre
 void launch_pivots(msmg_ctx* c, cudaStream_t s) {
   const Geo g = fine_geo(c);
   const size_t sm = (size_t)g.epc * (3 * g.P + g.nb) * sizeof(double);
-  cudaFuncSetAttribute(k_pivots, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  smem_at_least(k_pivots, sm);
   k_pivots<<<fine_grid(c, g), fine_threads(g), sm, s>>>(c->fine.T, c->n, g, c->fine.m, c->fine.nbr, c->fine.Wd,
                                                          c->fine.invd, c->fine.D, c->flags);
 }
@@ -319,7 +319,7 @@ void launch_faces_to_nat(msmg_ctx* c, double* out, cudaStream_t s) {
 void launch_matvec(msmg_ctx* c, const double* p, double* q, cudaStream_t s, int R) {
   const Geo g = fine_geo(c);
   const size_t sm = (size_t)g.epc * 4 * g.P * sizeof(double);
-  cudaFuncSetAttribute(k_matvec<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  smem_at_least(k_matvec<false>, sm);
   k_matvec<false><<<fine_grid(c, g) * R, fine_threads(g), sm, s>>>(p, q, c->fine.T, c->n, g, c->fine.m, c->fine.nbr,
                                                                     c->fine.Wd, c->red, nullptr, R);
 }

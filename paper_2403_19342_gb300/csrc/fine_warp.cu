@@ -2233,7 +2233,7 @@ static int resident_ctas(const void* k, int threads, size_t smem) {
 template <typename V, typename BT, typename G>
 static void prepare_t(msmg_ctx* c, const G& g) {
   auto smem = [](auto k, size_t bytes, bool carve) {
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    smem_at_least(k, bytes);
     if (carve) cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
   if constexpr (!IsCube8<G>::value) {

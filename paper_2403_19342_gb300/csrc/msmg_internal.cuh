@@ -16,6 +16,7 @@
 #include <cuda_bf16.h>
 #include <cstdint>
 #include <cstddef>
+#include <mutex>
 #include <vector>
 #include "../../include/msmg.h"
 
@@ -30,6 +31,18 @@ constexpr int kMaxLevels = MSMG_MAX_LEVELS;
     if (_e != cudaSuccess) { ::msmg::set_last_cuda_error(_e); return MSMG_ERR_CUDA; } \
   } while (0)
 void set_last_cuda_error(cudaError_t e);
+
+// Lets kernel k launch with `bytes` of dynamic shared memory.  The limit belongs to the
+// kernel and the device, not to a context, so it is only ever raised: a context with
+// larger elements, or a level with larger parents, may launch the same kernel later.
+template <typename K>
+inline void smem_at_least(K* k, size_t bytes) {
+  static std::mutex mu;   // set-ups on several threads: read and raise together
+  std::lock_guard<std::mutex> lock(mu);
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, k) == cudaSuccess && (size_t)a.maxDynamicSharedSizeBytes >= bytes) return;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
 
 // ---------------------------------------------------------------- arena
 // Bump allocator over the caller's workspace.  With base == nullptr it only

@@ -822,7 +822,7 @@ int launch_level1_eigen(msmg_ctx* c, cudaStream_t s) {
   FineLevel& f = c->fine;
   if (f.nb > 96) return MSMG_ERR_UNSUPPORTED;   // large elements use the subspace solver
   const size_t sm = jac_smem(f.nb, 2);
-  cudaFuncSetAttribute(k_eig_l1_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  smem_at_least(k_eig_l1_jacobi, sm);
   k_eig_l1_jacobi<<<(unsigned)f.m, 256, sm, s>>>(f.T, f.S, c->n, f.bx, f.by, f.bz, f.m, f.L, f.Phi, f.lam,
                                                   c->dtmp, f.Wd);
   return 0;
@@ -834,7 +834,7 @@ void launch_level1_galerkin(msmg_ctx* c, cudaStream_t s, bool threshold) {
   const double B = threshold ? c->opts.eig_threshold[0] : 0.0;
   k_level1_counts<<<(unsigned)((f.m + 7) / 8), 256, 0, s>>>(f.Phi, f.lam, f.m, f.L, f.nb, B, l2.cnt);
   const size_t sm = (size_t)(2 * f.L * f.nb + 3 * f.nb) * sizeof(double);
-  cudaFuncSetAttribute(k_galerkin1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  smem_at_least(k_galerkin1, sm);
   const unsigned thr = f.nb >= 256 ? 256 : (unsigned)((f.nb + 31) / 32 * 32 < 64 ? 64 : (f.nb + 31) / 32 * 32);
   k_galerkin1<<<(unsigned)f.m, thr, sm, s>>>(f.T, f.S, c->n, f.bx, f.by, f.bz, f.m, f.nbr, f.L, f.Phi, l2.Ad, l2.Ao,
                                              l2.F, l2.z, l2.cnt, f.Wd);
@@ -848,7 +848,7 @@ static int coarse_setup(msmg_ctx* c, int l, bool given, cudaStream_t s) {
   int tri = given ? 0 : tri_doubles(lv.nP, lv.Lnext);
   if (sm + (size_t)tri * sizeof(double) > 226 * 1024) tri = 0;
   sm += (size_t)tri * sizeof(double);
-  cudaFuncSetAttribute(k_coarse_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  smem_at_least(k_coarse_setup, sm);
   k_coarse_setup<<<(unsigned)lv.mP, 256, sm, s>>>(lv, nx, c->dtmp, given ? 1 : 0,
                                                   c->opts.coarse_smoother == MSMG_BLOCK_IC0,
                                                   given ? 0.0 : c->opts.eig_threshold[l - 1], tri);
