@@ -982,12 +982,14 @@ __global__ void __launch_bounds__(256) k_transpose_act(const TransArgs a) {
   }
 }
 
-// Adam (Kingma and Ba, 2015) on the FP32 masters; refresh the BF16 copies.
+// Adam (Kingma and Ba, 2015) on the FP32 masters; refresh the BF16 copies.  Nothing is
+// touched when the error word is set: the gradients are then incomplete (a product's wait
+// gave up), and masters and moments must survive the call that reports it.
 __global__ void k_adam(float* __restrict__ w, __nv_bfloat16* __restrict__ w16, const float* __restrict__ g,
                        float* __restrict__ m, float* __restrict__ v, int64_t n, float lr, float b1, float b2,
-                       float eps, float c1, float c2) {
+                       float eps, float c1, float c2, const int* __restrict__ err) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  if (i >= n || *err) return;
   const float gi = g[i];
   const float mi = b1 * m[i] + (1.f - b1) * gi;
   const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
@@ -1509,16 +1511,17 @@ int msmg_net_train_step(msmg_net* net, const float* x, const float* target, int 
   if (!net || !x || !target || batch < 1 || batch > net->d.batch_max || !(lr > 0.f)) return MSMG_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   net_backward(net, x, target, batch, net->grad, s);
-  net->step += 1;
+  if (net->map_err) return net_status(net, s);   // no product was launched: no gradients to step with
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float c1 = 1.f - powf(b1, (float)net->step), c2 = 1.f - powf(b2, (float)net->step);
+  const float k = (float)(net->step + 1), c1 = 1.f - powf(b1, k), c2 = 1.f - powf(b2, k);
   k_adam<<<g256(net->n_param), 256, 0, s>>>(net->w32, net->w16, net->grad, net->adam_m, net->adam_v, net->n_param, lr,
-                                            b1, b2, eps, c1, c2);
+                                            b1, b2, eps, c1, c2, net->err);
   net_refresh_bf16(net, s);
   {
     const int st = net_status(net, s, loss_host);
     if (st) return st;
   }
+  net->step += 1;
   if (loss_host) *loss_host /= (float)(batch * net->d.n_vec);
   MSMG_CUDA_TRY(cudaGetLastError());
   return 0;
