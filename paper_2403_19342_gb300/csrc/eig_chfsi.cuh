@@ -24,7 +24,8 @@
 // Gram-Schmidt.  K - L guard vectors keep the convergence rate set by the gap to
 // theta_{K-1}, not by clusters at the L-th eigenvalue.  The degree follows from the
 // reduction still needed: m = acosh(residual / tol) / acosh(t_L), 1 / T_m(t_L) being what
-// the filter leaves of the unwanted part of the L-th vector.
+// the filter leaves of the unwanted part of the L-th vector, and varies where the residual
+// does not fall (an unwanted eigenvalue at an extremum of T_m is not damped at all).
 //
 // Bound by the FP64 pipe (2 lanes per clock and SM).  Per cell and iteration, K = 10:
 // filter 7 K per degree, A~ X 70, G and H 55 each with 14 of reduction, rotation and
@@ -537,8 +538,8 @@ __global__ void __launch_bounds__(kEigThreads) k_eig_l1_chfsi(const double* __re
   }
   const double bup = misc[0];
 
-  int it = 0, stall = 0;
-  double rmax = 0.0, rbest = 1e300;
+  int it = 0, stall = 0, slow = 0;
+  double rmax = 0.0, rbest = 1e300, rprev = 1e300;
   for (;; ++it) {
     for (int attempt = 0; attempt < 2; ++attempt) {
       // ---- Y = A~ X
@@ -633,6 +634,15 @@ __global__ void __launch_bounds__(kEigThreads) k_eig_l1_chfsi(const double* __re
         const double d = fmin(ceil(need / al), fmin(top, fmax(keep, 10.0)));
         deg = d >= 4.0 ? (int)d : 4;
       }
+      // Where an iteration leaves more than half of the residual, every second one takes
+      // 1, 3 or 5 degrees less.  On a cluster at the cutoff the interval and so the degree
+      // settle, and an unwanted eigenvalue inside the interval at an extremum of that T_m
+      // keeps its part of the block from one iteration to the next: a four-layer element
+      // below a channel of 4.7e7 (L = 12) took 260 iterations, 1000 and more from some
+      // starting blocks; with the degree varied 16 and 61.  Elements without such a
+      // cluster halve their residual every time and are not touched.
+      if (rmax > 0.5 * rprev && (++slow & 1)) deg = deg - slow % 6 > 4 ? deg - slow % 6 : 4;
+      rprev = rmax;
       misc[2] = (double)deg;
     }
     __syncthreads();
