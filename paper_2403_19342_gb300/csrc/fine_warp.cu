@@ -1,6 +1,6 @@
 // Fine-level PCG iteration kernels.  Two sets: one warp per element (two in the FP64
-// k_post on 8^3 elements, see elem_threads), which 8^3 elements and small FP64 grids
-// take, and groups of elements per CTA (the k_*_grp kernels, use_groups) for the rest.
+// k_post on 8^3 elements, see elem_threads), which 8^3 and other large elements and small
+// FP64 grids take, and groups of elements per CTA (the k_*_grp kernels, use_groups).
 //
 // In the first set each element of E_1 (bx x by x bz cells) is handled by one warp.  Its data is
 // one contiguous chunk of every block-major array; the warp stages what it
@@ -1339,19 +1339,20 @@ __global__ void __launch_bounds__(kPmWarps * 32, kPmCtasPerSm) k_pmatvec(const d
 
 // ------------------------------------------------------------------ groups of elements
 // The fine kernels on groups of consecutive elements, E per CTA of 128 threads (E by <=
-// 32), for elements smaller than 8^3 (use_groups).  Latency and issue bind them.  The
-// group's cells are one contiguous range of every array, which all threads stream (a warp
-// per 80-cell element left lanes idle and its unrolled loops mostly predicated off); the
+// 32), for small elements (use_groups).  Latency and issue bind them.  The group's
+// cells are one contiguous range of every array, which all threads stream (a warp per
+// 80-cell element left lanes idle and its unrolled loops mostly predicated off); the
 // IC(0) sweeps are run by one warp, a lane per (element, ly): lane (e, ly) walks its
-// x-lines lz = 0 .. bz-1, one per step s = ly + lz, keeping the line in registers.  The line's neighbours are its own previous line (lz - 1) and the previous line
-// of the lane before it (ly - 1, by shuffle), so a sweep of an 8^3 element is 15 steps of
-// 8 cells without a barrier, and reads shared memory in 16-byte pieces: 14 instructions a
-// step for four elements.  Per cell the arithmetic and its order are those of w_ic0_s.
+// x-lines lz = 0 .. bz-1, one per step s = ly + lz, keeping the line in registers.  The
+// line's neighbours are its own previous line (lz - 1) and the previous line of the lane
+// before it (ly - 1, by shuffle), so a sweep of an 8 x 8 x 4 element is 11 steps of 8 cells
+// without a barrier, and reads shared memory in 16-byte pieces: 14 instructions a step for
+// four elements.  Per cell the arithmetic and its order are those of w_ic0_s.
 // 60 x 220 x 85 cells, 4 x 4 x 5 elements, mixed (event times, us): pre 76 -> 39, post
 // 132 -> 56, restrict 61 -> 47, pmatvec 65 -> 48.  On 8^3 elements the same kernels are
 // slower than a warp per element (128^3: post 63 against 51; 256^3: pre 279 against 262:
 // the sweeping warp's chains are four times longer and the rest of the CTA waits for
-// them), so those keep theirs.
+// them), so those and, kernel by kernel, other large ones keep theirs.
 // Shared memory holds the planes of an element PP apart (a multiple of 32 words gets 4
 // more: lanes of one element are then on different banks), elements EP = PP bz apart.
 constexpr int kGThreads = 128;
@@ -2084,17 +2085,38 @@ static inline unsigned fine_wgrid(const msmg_ctx* c, int W = kWarpsPerCta) {
   return (unsigned)((c->fine.m + W - 1) / W * c->sb.R);
 }
 
-// a warp per element is compiled for every shape but FP32 4^3 elements, which always take groups
-template <typename V, typename G>
-constexpr bool kHasWarp = !(std::is_same<V, float>::value && std::is_same<G, GeoC<4, 4, 4>>::value);
-// Groups of elements: where a warp has a lane for every x-line of a z-plane, except 8^3
-// elements, and in FP64 except grids of few elements (a sweeping warp's FP64 chains take
-// twice as long as a warp per element's, which shows where all elements run at once:
-// 512 elements of 4^3, a solve 1.13 against 1.39 ms).
-template <typename V, typename G>
+// Which kernels take groups: by element size, since an element that fills its own warp's
+// lanes gains less while the sweeping warp's chains and the shared memory of E elements
+// grow.  1 to 1.7 M cells, us, a warp per element / groups (one right-hand side):
+//   FP32 pre    4x4x5 96 / 43, 6x6x6 73 / 43, 8x8x6 70 / 49; 4^3 40 / 42; lines of 12 to 16:
+//               16x2x2 143 / 47, 16x8x4 63 / 76
+//   FP32 post   4x4x5 164 / 59, 6x6x6 110 / 92, 8x8x4 94 / 65; 6x6x8 91 / 112, 7x7x7 99 / 113;
+//               lines of 5 and 7, swept out of shared memory: 5x5x5 144 / 113, 5x5x8 110 / 116
+//   FP64 pre    4x4x5 149 / 76, 6x6x6 108 / 88; 8x8x4 92 / 108, 8x8x6 99 / 167
+//   FP64 post   4x4x5 285 / 138, 4x6x6 214 / 153; 6x6x6 187 / 197, 8x8x4 167 / 266
+//   pmatvec     4x4x5 80 / 53, 6x6x6 55 / 46, 8x8x4 58 / 57; 8x8x6 49 / 50
+//   restrict    4x4x5 FP32 74 / 52, FP64 174 / 106; 8x8x6 56 / 37 and 157 / 98
+// Lines above 8 keep groups up to 96 cells (FP64 post 12x2x4 261 / 211; 12x4x4 171 / 213).  Long thin
+// elements are mostly halo, and one with more than 16 y-lines is a group alone: 2x32x2 pre
+// 192 / 271; 2x2x32 pmatvec 60 / 97, FP64 post 331 / 384, FP64 restrict 133 / 164.  FP64 takes
+// groups from 16 elements per SM: a sweeping warp's FP64 chains take twice as long as a warp
+// per element's, which shows where all elements run at once (512 elements of 4^3, a solve
+// 1.13 against 1.39 ms); the restriction likewise (288 elements of 4x4x5, three right-hand
+// sides: 14 against 16 us).
+enum GrpKernel { kGrpPre, kGrpRestrict, kGrpPost, kGrpPmatvec };
+template <GrpKernel K, typename V, typename G>
 static bool use_groups(const msmg_ctx* c, const G& g) {
-  return !IsCube8<G>::value && g.by <= 32 && (sizeof(V) == 4 || c->fine.m >= 152 * 16);
+  const bool f32 = sizeof(V) == 4, many = c->fine.m >= 152 * 16;
+  if (IsCube8<G>::value || g.by > 16 || (!f32 && !many)) return false;
+  auto up_to = [&](int cells) { return g.nb <= (g.bx <= 8 ? cells : 96); };
+  if (K == kGrpPre) return f32 ? up_to(512) && !IsGeoC<G>::value : up_to(216);
+  if (K == kGrpPost) return f32 ? up_to(g.bx == 5 || g.bx == 7 ? 128 : 256) : up_to(144) && g.bz <= 16;
+  if (K == kGrpPmatvec) return up_to(256) && g.by <= 12 && g.bz <= 12;
+  return many && !IsGeoC<G>::value && (f32 || g.bz <= 16);   // restrict: not on 4^3, two full cells a lane
 }
+// the warp kernels that no element reaches are not compiled
+template <typename V, typename G>
+constexpr bool kHasWarpPost = !(std::is_same<V, float>::value && std::is_same<G, GeoC<4, 4, 4>>::value);
 template <typename G>
 static unsigned grp_grid(const msmg_ctx* c, const G& g) {
   const int E = make_grp(g).E;
@@ -2121,29 +2143,24 @@ template <typename V, typename BT, typename G>
 static void pre_t(msmg_ctx* c, const FineOps<V, BT>& o, int update, PcgScalars* sc, cudaStream_t s, const G& g) {
   SolveBuffers& B = c->sb;
   if constexpr (!IsCube8<G>::value) {
-    if (use_groups<V>(c, g)) {
+    if (use_groups<kGrpPre, V>(c, g)) {
       k_pre_grp<V, G><<<grp_grid(c, g), kGThreads, grp_pre_floats(g) * sizeof(V), s>>>(
           B.x, B.r, B.pcur, B.q, o.T, o.invd, (V*)B.rv, (V*)B.vu[1], c->n, g, c->fine.m, update, c->red, sc,
           c->flags + 6, B.R);
       return;
     }
   }
-  if constexpr (kHasWarp<V, G>) {
-    constexpr int W = stage_elems<kStagePre, V, G>();
-    k_pre<V, G><<<fine_wgrid(c, W), W * elem_threads<kStagePre, G, V>(), wsmem<kStagePre, V>(g), s>>>(
-        B.x, B.r, B.pcur, B.q, o.T, o.invd, (V*)B.rv, (V*)B.vu[1], c->n, g, c->fine.m, c->fine.nbr, update, c->red, sc,
-        c->flags + 6, B.R);
-  }
+  constexpr int W = stage_elems<kStagePre, V, G>();
+  k_pre<V, G><<<fine_wgrid(c, W), W * elem_threads<kStagePre, G, V>(), wsmem<kStagePre, V>(g), s>>>(
+      B.x, B.r, B.pcur, B.q, o.T, o.invd, (V*)B.rv, (V*)B.vu[1], c->n, g, c->fine.m, c->fine.nbr, update, c->red, sc,
+      c->flags + 6, B.R);
 }
 
 template <typename V, typename BT, typename G>
 static void restrict_t(msmg_ctx* c, const FineOps<V, BT>& o, PcgScalars* sc, cudaStream_t s, const G& g) {
   SolveBuffers& B = c->sb;
-  // groups only from 16 elements per SM (60 x 220 x 85: 61 -> 47 us; 288 elements of 4 x 4 x 5,
-  // three right-hand sides: 14 -> 16), and not on 4^3, whose warps have two full cells a lane
-  // (72 x 48 x 104: 12.2 against 14.2 us)
   if constexpr (!IsGeoC<G>::value) {
-    if (use_groups<V>(c, g) && c->fine.m >= 152 * 16) {
+    if (use_groups<kGrpRestrict, V>(c, g)) {
       k_restrict_grp<V, BT, G><<<grp_grid(c, g), kGThreads, grp_tile_bytes(g, sizeof(V), true), s>>>(
           (const V*)B.rv, (const V*)B.vu[1], o.T, o.Wd, o.Phi, c->fine.L, (double*)B.vf[2], c->lev[2].n, c->n, g,
           c->fine.m, c->fine.nbr, sc, B.R);
@@ -2161,7 +2178,7 @@ static void post_t(msmg_ctx* c, const FineOps<V, BT>& o, const V* ec, const doub
                    cudaStream_t s, const G& g, bool fuse) {
   SolveBuffers& B = c->sb;
   if constexpr (!IsCube8<G>::value) {
-    if (use_groups<V>(c, g)) {
+    if (use_groups<kGrpPost, V>(c, g)) {
       auto run = [&](auto k, int pf) {
         k<<<grp_grid(c, g), kGThreads, grp_post_floats(g) * sizeof(V), s>>>(
             (const V*)B.rv, B.r, (const V*)B.vu[1], o.T, o.Wd, o.invd, o.Phi, ec, c->fine.L, c->lev[2].n, B.z, qv,
@@ -2173,7 +2190,7 @@ static void post_t(msmg_ctx* c, const FineOps<V, BT>& o, const V* ec, const doub
       return;
     }
   }
-  if constexpr (kHasWarp<V, G>) {
+  if constexpr (kHasWarpPost<V, G>) {
     constexpr int W = stage_elems<kStageFull, V, G>();
     constexpr int NT = elem_threads<kStageFull, G, V>();
     if (fuse)
@@ -2206,7 +2223,7 @@ template <typename G>
 static void pmatvec_t(msmg_ctx* c, PcgScalars* sc, cudaStream_t s, const G& g) {
   SolveBuffers& B = c->sb;
   if constexpr (!IsCube8<G>::value) {
-    if (use_groups<double>(c, g)) {
+    if (use_groups<kGrpPmatvec, double>(c, g)) {
       k_pmatvec_grp<G><<<grp_grid(c, g), kGThreads, grp_tile_bytes(g, sizeof(double), false), s>>>(
           B.z, B.pcur, B.pnext, B.q, c->fine.T, c->fine.D, c->n, g, c->fine.m, c->fine.nbr, c->red, sc, B.R);
       return;
@@ -2237,10 +2254,11 @@ static void prepare_t(msmg_ctx* c, const G& g) {
     if (carve) cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
   };
   if constexpr (!IsCube8<G>::value) {
-    if (use_groups<double>(c, g)) smem(k_pmatvec_grp<G>, grp_tile_bytes(g, sizeof(double), false), true);
-    if (use_groups<V>(c, g)) {
-      smem(k_pre_grp<V, G>, grp_pre_floats(g) * sizeof(V), true);
-      if constexpr (!IsGeoC<G>::value) smem(k_restrict_grp<V, BT, G>, grp_tile_bytes(g, sizeof(V), true), true);
+    if (use_groups<kGrpPmatvec, double>(c, g)) smem(k_pmatvec_grp<G>, grp_tile_bytes(g, sizeof(double), false), true);
+    if (use_groups<kGrpPre, V>(c, g)) smem(k_pre_grp<V, G>, grp_pre_floats(g) * sizeof(V), true);
+    if constexpr (!IsGeoC<G>::value)
+      if (use_groups<kGrpRestrict, V>(c, g)) smem(k_restrict_grp<V, BT, G>, grp_tile_bytes(g, sizeof(V), true), true);
+    if (use_groups<kGrpPost, V>(c, g)) {
       const size_t so = grp_post_floats(g) * sizeof(V);
       auto post = [&](auto k, int i) {
         smem(k, so, true);
@@ -2252,10 +2270,10 @@ static void prepare_t(msmg_ctx* c, const G& g) {
   }
   smem(k_pmatvec<G>, wsmem_p(g), true);
   smem(k_restrict<V, BT, G>, wsmem<restrict_layout<V>(), V>(g), true);
-  if constexpr (kHasWarp<V, G>) {
-    if (!use_groups<V>(c, g)) {
+  smem(k_pre<V, G>, wsmem<kStagePre, V>(g), false);
+  if constexpr (kHasWarpPost<V, G>) {
+    if (!use_groups<kGrpPost, V>(c, g)) {
       const size_t smv = wsmem<kStageFull, V>(g);
-      smem(k_pre<V, G>, wsmem<kStagePre, V>(g), false);
       smem(k_post<V, BT, G, true>, smv, true);
       smem(k_post<V, BT, G, false>, smv, true);
       constexpr int NT = elem_threads<kStageFull, G, V>();
