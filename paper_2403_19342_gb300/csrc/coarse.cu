@@ -66,20 +66,13 @@ struct LevelData {
   const S *Ad, *Ao, *Minv, *Psi;
 };
 
-// Loads of f and u: through the read-only path when they were written by an
-// earlier launch (per-level kernels), coherent when an earlier phase of the same
-// launch wrote them (the fused forms, the inner two-grid solve).
-template <bool NC, typename S>
-__device__ __forceinline__ S ld_vec(const S* p) {
-  if constexpr (NC) return __ldg(p);
-  else return *p;
-}
-
 // Partial s of r_i = f_i - (A_l u)_i for row t of parent P: s = 0 takes f and
 // the element's own block, s = 1, 2, 3 its x, y, z neighbour blocks (+d, then
 // -d).  The row is (p0 + p1) + (p2 + p3): four threads (per-level kernels) or
-// one thread in turn (fused forms) give the same bits.
-template <int LT, typename S, bool NC = true>
+// one thread in turn (fused forms) give the same bits.  f and u were written by an earlier
+// phase of the launch or by a launch that may still run when this one starts: plain loads,
+// never the read-only path.
+template <int LT, typename S>
 __device__ __forceinline__ S coarse_residual_part(const CoarseLevel& lv, const LevelData<S>& D, int64_t P, int t,
                                                   int s, const S* f, const S* u) {
   const int L = LT ? LT : lv.L;
@@ -89,12 +82,12 @@ __device__ __forceinline__ S coarse_residual_part(const CoarseLevel& lv, const L
   if (s == 0) {
     const S* ad = D.Ad + a * L2 + (size_t)k * L;
     const S* ua = u + a * L;
-    S acc = ld_vec<NC>(f + a * L + k);
+    S acc = f[a * L + k];
     if (LT) {
 #pragma unroll
-      for (int mm = 0; mm < LT; ++mm) acc -= __ldg(ad + mm) * ld_vec<NC>(ua + mm);
+      for (int mm = 0; mm < LT; ++mm) acc -= __ldg(ad + mm) * ua[mm];
     } else {
-      for (int mm = 0; mm < L; ++mm) acc -= __ldg(ad + mm) * ld_vec<NC>(ua + mm);
+      for (int mm = 0; mm < L; ++mm) acc -= __ldg(ad + mm) * ua[mm];
     }
     return acc;
   }
@@ -107,9 +100,9 @@ __device__ __forceinline__ S coarse_residual_part(const CoarseLevel& lv, const L
     const S* ub = u + (int64_t)bp * L;
     if (LT) {
 #pragma unroll
-      for (int mm = 0; mm < LT; ++mm) acc -= __ldg(ao + mm) * ld_vec<NC>(ub + mm);
+      for (int mm = 0; mm < LT; ++mm) acc -= __ldg(ao + mm) * ub[mm];
     } else {
-      for (int mm = 0; mm < L; ++mm) acc -= __ldg(ao + mm) * ld_vec<NC>(ub + mm);
+      for (int mm = 0; mm < L; ++mm) acc -= __ldg(ao + mm) * ub[mm];
     }
   }
   if (bm >= 0) {
@@ -117,21 +110,21 @@ __device__ __forceinline__ S coarse_residual_part(const CoarseLevel& lv, const L
     const S* ub = u + (int64_t)bm * L;
     if (LT) {
 #pragma unroll
-      for (int mm = 0; mm < LT; ++mm) acc -= __ldg(ao + (size_t)mm * LT) * ld_vec<NC>(ub + mm);
+      for (int mm = 0; mm < LT; ++mm) acc -= __ldg(ao + (size_t)mm * LT) * ub[mm];
     } else {
-      for (int mm = 0; mm < L; ++mm) acc -= __ldg(ao + (size_t)mm * L) * ld_vec<NC>(ub + mm);
+      for (int mm = 0; mm < L; ++mm) acc -= __ldg(ao + (size_t)mm * L) * ub[mm];
     }
   }
   return acc;
 }
 
-template <int LT, typename S, bool NC = true>
+template <int LT, typename S>
 __device__ __forceinline__ S coarse_residual_row(const CoarseLevel& lv, const LevelData<S>& D, int64_t P, int t,
                                                  const S* f, const S* u) {
-  const S p0 = coarse_residual_part<LT, S, NC>(lv, D, P, t, 0, f, u);
-  const S p1 = coarse_residual_part<LT, S, NC>(lv, D, P, t, 1, f, u);
-  const S p2 = coarse_residual_part<LT, S, NC>(lv, D, P, t, 2, f, u);
-  const S p3 = coarse_residual_part<LT, S, NC>(lv, D, P, t, 3, f, u);
+  const S p0 = coarse_residual_part<LT, S>(lv, D, P, t, 0, f, u);
+  const S p1 = coarse_residual_part<LT, S>(lv, D, P, t, 1, f, u);
+  const S p2 = coarse_residual_part<LT, S>(lv, D, P, t, 2, f, u);
+  const S p3 = coarse_residual_part<LT, S>(lv, D, P, t, 3, f, u);
   return (p0 + p1) + (p2 + p3);
 }
 
@@ -333,7 +326,7 @@ __global__ void k_coarse_resid_restrict(CoarseLevel lv, LevelData<S> D, const S*
     q = quad_combine(q);
     if (row < nP && (t & 3) == 0) rs[row] = q;
   } else {
-    if (t < nP) rs[t] = coarse_residual_row<LT, S, false>(lv, D, P, t, f, u);
+    if (t < nP) rs[t] = coarse_residual_row<LT, S>(lv, D, P, t, f, u);
   }
   cp_wait();
   __syncthreads();
@@ -424,7 +417,7 @@ __global__ void k_coarse_resid_smooth(CoarseLevel lv, LevelData<S> D, const S* f
       if (out32) out32[P * nP + row] = (float)v;
     }
   } else {
-    if (t < nP) rs[t] = coarse_residual_row<LT, S, false>(lv, D, P, t, f, u);
+    if (t < nP) rs[t] = coarse_residual_row<LT, S>(lv, D, P, t, f, u);
     cp_wait();
     __syncthreads();
     if (t < nP) {
@@ -604,7 +597,7 @@ __device__ void tail_level_down(const TailArgs& A, int l, int r0, int r1, int ct
     const double* f = A.f[l] + (int64_t)it.r * lv.n;
     const double* u = A.u[l] + (int64_t)it.r * lv.n;
     double* fn = A.f[l + 1] + (int64_t)it.r * lv.mP * Ln;
-    const double rt = (live && t < nP) ? coarse_residual_row<LT, double, false>(lv, D, it.P, t, f, u) : 0.0;
+    const double rt = (live && t < nP) ? coarse_residual_row<LT, double>(lv, D, it.P, t, f, u) : 0.0;
     double* red = fs + nP;
     for (int j = 0; j < Ln; ++j) {
       double v = (live && t < nP) ? __ldg(D.Psi + ((size_t)it.P * Ln + j) * nP + t) * rt : 0.0;
@@ -659,7 +652,7 @@ __device__ void tail_level_up(const TailArgs& A, int l, int r0, int r1, int cta,
     double* w = A.w[l] + (int64_t)it.r * lv.n;
     float* o32 = (l == 2 && A.out32) ? A.out32 + (int64_t)it.r * lv.n : nullptr;
     if (live) group_cp(Mi, D.Minv + (size_t)it.P * nP * nP, nP * nP, t, gw * 32);
-    if (live && t < nP) rs[t] = coarse_residual_row<LT, double, false>(lv, D, it.P, t, f, u);
+    if (live && t < nP) rs[t] = coarse_residual_row<LT, double>(lv, D, it.P, t, f, u);
     cp_wait();
     __syncthreads();
     if (live && t < nP) {

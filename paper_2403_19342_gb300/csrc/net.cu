@@ -46,8 +46,8 @@ struct msmg_net {
   __nv_bfloat16* xb;            // [batch_max][n_in] BF16 input (the products' A operand)
   __nv_bfloat16* h1b;           // [batch_max][h1] BF16 activations
   __nv_bfloat16* h2b;           // [batch_max][h2]
-  // backward (chunks of at most rc rows, rcp = rc rounded up to 64)
-  int rc, rcp;
+  // backward (chunks of at most rc rows; rcp: rc rounded up to 64)
+  int rc;
   __nv_bfloat16* dk;            // [3][rc][ldk] BF16 parts of a layer's output gradient
   __nv_bfloat16* dt;            // [3][fan_out][rcp] the same transposed, zero beyond the rows
   __nv_bfloat16* at[3];         // [fan_in][rcp] transposed BF16 input of each layer, zero beyond the rows
@@ -1285,7 +1285,7 @@ static int64_t net_carve(const msmg_net_desc* d, Arena& ar, msmg_net* t) {
     t->wgt = wgt;
     t->step = 0;
     t->wt16 = wt16; t->xb = xb; t->h1b = h1b; t->h2b = h2b; t->err = err;
-    t->rc = (int)rc; t->rcp = (int)rcp;
+    t->rc = (int)rc;
     t->dk = dk; t->dt = dt; t->part = part; t->part_cap = part_cap;
     for (int l = 0; l < 3; ++l) { t->at[l] = at[l]; t->csum[l] = csum[l]; t->wp[l] = wp[l]; t->ldw[l] = ldw[l]; }
     t->tc = tc;
