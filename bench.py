@@ -687,7 +687,10 @@ def run_layered(args, world, rank, local):
     for name, ws in (("cold", None), ("warm", net)):
         S = pkg.Solver(kappa, pkg.Options(**base, warm_start=ws))
         i = S.info
-        recs[name] = {"setup_ms": i["setup_ms"], "eig_ms": i["eig_ms"], "eig_iterations_total": i["eig_iterations_total"],
+        if S.setup_status != 0:
+            raise RuntimeError(f"{name} set-up: status {S.setup_status}, eigenresidual {i['eig_residual_max']:.3g} "
+                               f"after {i['eig_iterations_max']} iterations")
+        recs[name] = {"setup_status": S.setup_status, "setup_ms": i["setup_ms"], "eig_ms": i["eig_ms"], "eig_iterations_total": i["eig_iterations_total"],
                       "eig_iterations_max": i["eig_iterations_max"], "eig_residual_max": i["eig_residual_max"],
                       "warm_started": i["warm_started"]}
         if name == "warm":
