@@ -403,11 +403,11 @@ int msmg_setup(const msmg_grid* grid, const void* kappa, int kappa_components, i
   cudaEventCreate(&c->ev0);
   cudaEventCreate(&c->ev1);
   // untuned defaults: separate prolongation and a launch per coarse step, the fastest of the
-  // variants on every hierarchy they were timed on (us per iteration, these / the fused
-  // prolongation / the cooperative coarse cycle: 32^3 FP64 76 / 78 / 91, 96^3 FP64
-  // 298 / 317 / 328, 256^3 mixed 1297 / 1351 / 1366, 60x220x85 with wells 423 / 501 / 477,
-  // 96^3 with 16 right-hand sides 969 / 1013 / 996; since then the launches overlap and
-  // groups of elements came: 72, 295, 1288, 271 and 966)
+  // variants on every hierarchy and width they were timed on (us per iteration of a solve,
+  // these / the fused prolongation / the cooperative coarse cycle: 32^3 FP64 58 / 62 / 76,
+  // with 16 right-hand sides 235 / 256 / 248; 64^3 mixed 81 / 84 / 99; 96^3 FP64
+  // 282 / 301 / 313; 128^3 mixed 231 / 244 / 280, 16 right-hand sides 2251 / 2385 / 2341;
+  // 256^3 mixed 1281 / 1335 / 1352; 60x220x85 with wells 266 / 456 / 327)
   c->tune_fused[0] = c->tune_fused[1] = 0;
   c->tune_tail[0] = c->tune_tail[1] = 0;
   for (int k = 0; k < 3; ++k) cudaEventCreateWithFlags(&c->poll_evs[k], cudaEventDisableTiming);

@@ -261,7 +261,11 @@ __host__ __device__ inline unsigned coarse_threads4_d(int nP, int Ln) {
 // one-path residuals and the four sums at a time below, 128^3 coarse levels 70 -> 47 us
 // launched singly, a whole iteration in the graph 232 -> 225; 32^3 75 -> 72;
 // 60 x 220 x 85 278 -> 271.  Letting the fine restriction start the first coarse launch
-// as well cost 72 x 48 x 104 8 us, so that one waits for its end.
+// as well cost 72 x 48 x 104 8 us, so that one waits for its end.  The overlap by itself
+// (us per iteration without / with): one right-hand side 32^3 59.5 / 57.9, 96^3 124.2 / 122.2,
+// 128^3 235.0 / 231.0, 60 x 220 x 85 270.7 / 266.3; several, where the CTAs fill the GPU
+// and there is little to overlap, within 1.2% either way: 128^3 x 3 531 / 536,
+// 64^3 x 4 117.3 / 115.9, 96^3 x 16 964 / 961, 128^3 x 16 2256 / 2251.
 
 // Row layouts of the per-level kernels, the same bits either way: QUAD, four
 // threads per row (a level with few parents: shorter dependent chains, more
