@@ -68,8 +68,7 @@ namespace msmg {
 // ------------------------------------------------------------------ CUDA-core product
 // C = epi(A[M][K] B[K][N] + bias), BF16 operands, FP32 accumulation, for the forward
 // pass of networks whose widths are not multiples of 64.  Each output is one chain of
-// fmaf over k = 0 .. K-1, whatever the tile.  256 threads (64 for the smallest tile),
-// TM x TN outputs each; the next K block is in registers while this one is multiplied.
+// fmaf over k = 0 .. K-1, whatever the tile.  256 threads, TM x TN outputs each; the next K block is in registers while this one is multiplied.
 //   EPI 2: ReLU, stored in BF16 (the next layer's operand); EPI 3: times wgt[m][n mod n_in], FP32.
 template <int BM, int BN, int BK, int TM, int TN, int EPI>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
@@ -144,15 +143,16 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN))
 }
 
 static int sm_count();
-// The largest of three tiles that still gives most SMs one (a smaller tile re-reads more
-// of its operands, a larger one leaves SMs idle).
+// 64 x 64 tiles where every SM gets one, 32 x 32 below that (512 -> 1000 -> 1000 -> 2560,
+// 50 rows 193 -> 122 us, 300 rows 215 against 230).  128 x 128 tiles gain at most 5% where
+// their number happens to fill the SMs evenly and lose up to 27% where it does not (64 / 128,
+// us: 3000 rows of 216 -> 450 -> 900 -> 864 352 / 449, of 512 -> 1000 -> 1000 -> 2560
+// 835 / 968, 8192 rows of it 2108 / 2089), so there are none.
 template <int EPI>
 static void gemm(const __nv_bfloat16* A, const __nv_bfloat16* B, float* C, __nv_bfloat16* Cb, const float* bias,
                  const float* wgt, int n_in, int M, int N, int K, cudaStream_t s) {
   auto tiles = [&](int bm, int bn) { return (int64_t)((M + bm - 1) / bm) * ((N + bn - 1) / bn); };
-  if (tiles(128, 128) >= sm_count())
-    k_gemm<128, 128, 16, 8, 8, EPI><<<dim3((N + 127) / 128, (M + 127) / 128), 256, 0, s>>>(A, B, C, Cb, bias, wgt, n_in, M, N, K);
-  else if (tiles(64, 64) >= sm_count())
+  if (tiles(64, 64) >= sm_count())
     k_gemm<64, 64, 32, 4, 4, EPI><<<dim3((N + 63) / 64, (M + 63) / 64), 256, 0, s>>>(A, B, C, Cb, bias, wgt, n_in, M, N, K);
   else
     k_gemm<32, 32, 32, 2, 2, EPI><<<dim3((N + 31) / 32, (M + 31) / 32), 256, 0, s>>>(A, B, C, Cb, bias, wgt, n_in, M, N, K);
