@@ -1212,8 +1212,46 @@ static const double* launch_inner(msmg_ctx* c, PcgScalars* sc, cudaStream_t s) {
 
 // Shared-memory limits of the coarse kernels and the fused forms (set once per
 // context, never during capture).
+// registers a CTA of the kernel holds on its SM (allocated per warp in units of 256)
+template <typename K>
+static int cta_regs(K* k, unsigned threads) {
+  cudaFuncAttributes a;
+  if (cudaFuncGetAttributes(&a, k) != cudaSuccess) return 65536;
+  return (a.numRegs * 32 + 255) / 256 * 256 * (int)((threads + 31) / 32);
+}
+
+// Whether the coarsest GEMV (grid CTAs of 256) starts while the restriction before it runs.
+// Started early, its CTAs go beside that launch's; where only some of them fit, the rest land
+// later on whichever SMs are free first, on top of those, and such an SM takes a third longer
+// than with the even spread of a launch by itself (128^3, L = 7: 448 CTAs, 400 fit: coarse
+// levels 96 us overlapped, 72 not; L = 6: 384 fit: 55 against 61).  More CTAs than the GPU
+// holds at once even out (128^3 with 16 kept, 1024 CTAs: 175 against 185).
+static bool gemv_overlaps(const msmg_ctx* c, int64_t grid) {
+  if (c->nL == 2) return true;           // follows a fine kernel, which starts nothing early
+  constexpr int kRegs = 65536, kThreads = 2048, kSms = 152;
+  const CoarseLevel& lv = c->lev[c->nL - 1];
+  const int64_t before = lv.mP * c->sb.R;
+  const bool quad = before < kSms * 8;
+  const int64_t regs = c->restrict_regs[quad], thr = quad ? coarse_threads4(lv) : coarse_threads(lv);
+  auto room = [&](int64_t k) {           // CTAs that fit beside k of the launch before
+    const int64_t a = (kRegs - k * regs) / c->gemv_regs, b = (kThreads - k * thr) / 256, r = a < b ? a : b;
+    return r > 0 ? r : (int64_t)0;
+  };
+  const int64_t k = before / kSms, more = before % kSms;
+  return grid > kSms * room(0) || grid <= room(k) * (kSms - more) + room(k + 1) * more;
+}
+
 void prepare_coarse_kernels(msmg_ctx* c) {
   prepare_t<double>(c);
+  c->gemv_regs = cta_regs(k_dense_gemv<double>, 256);
+  if (c->nL > 2) {
+    const CoarseLevel& lv = c->lev[c->nL - 1];
+    with_L(lv.L, [&](auto LC) {
+      constexpr int LT = decltype(LC)::value;
+      c->restrict_regs[0] = cta_regs(k_coarse_resid_restrict<LT, double, false>, coarse_threads(lv));
+      c->restrict_regs[1] = cta_regs(k_coarse_resid_restrict<LT, double, true>, coarse_threads4(lv));
+    });
+  }
   tail_prepare(c);
   c->inner_grid = 0;
   if (c->opts.two_grid && c->nL >= 3 && c->coop_smem)
@@ -1273,8 +1311,11 @@ static const S* coarse_cycle_t(msmg_ctx* c, int l, PcgScalars* sc, cudaStream_t 
   }
   if (l == c->nL) {
     const unsigned grid = (unsigned)((lv.n * 32 + 255) / 256 * R);
-    launch_next(k_dense_gemv<S>, grid, 256, 0, s, lv.pinv, f, u, l == 2 ? c->sb.ec32 : nullptr, lv.n, lv.nk, lv.cmap,
-                lv.cinv, sc, R);
+    float* o32 = l == 2 ? c->sb.ec32 : nullptr;
+    if (gemv_overlaps(c, grid))
+      launch_next(k_dense_gemv<S>, grid, 256, 0, s, lv.pinv, f, u, o32, lv.n, lv.nk, lv.cmap, lv.cinv, sc, R);
+    else
+      k_dense_gemv<S><<<grid, 256, 0, s>>>(lv.pinv, f, u, o32, lv.n, lv.nk, lv.cmap, lv.cinv, sc, R);
     return u;
   }
   const LevelData<S> D = level_data<S>(lv);

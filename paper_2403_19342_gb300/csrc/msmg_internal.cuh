@@ -235,6 +235,7 @@ struct msmg_ctx {
   int tail_lt;                                  // compile-time L of the tail levels (0: runtime)
   size_t tail_smem;
   int coop_grid;                                // CTAs of the cooperative coarse cycle (0: unavailable)
+  int gemv_regs, restrict_regs[2];              // registers of a CTA: the coarsest GEMV, the restriction to it (one thread, four per row)
   int inner_grid;                               // CTAs of the exact two-grid inner solve (0: unavailable)
   unsigned long long* kept;                     // [kMaxLevels + 1] sum of cnt per level (device)
   int* cmaps;                                   // [2 n_L] storage of the coarsest packing maps
