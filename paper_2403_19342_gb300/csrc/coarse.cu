@@ -265,7 +265,8 @@ __host__ __device__ inline unsigned coarse_threads4_d(int nP, int Ln) {
 // (us per iteration without / with): one right-hand side 32^3 59.5 / 57.9, 96^3 124.2 / 122.2,
 // 128^3 235.0 / 231.0, 60 x 220 x 85 270.7 / 266.3; several, where the CTAs fill the GPU
 // and there is little to overlap, within 1.2% either way: 128^3 x 3 531 / 536,
-// 64^3 x 4 117.3 / 115.9, 96^3 x 16 964 / 961, 128^3 x 16 2256 / 2251.
+// 64^3 x 4 117.3 / 115.9, 96^3 x 16 964 / 961, 128^3 x 16 2256 / 2251.  The coarsest GEMV,
+// which streams its matrix, overlaps only where it fits (gemv_overlaps).
 
 // Row layouts of the per-level kernels, the same bits either way: QUAD, four
 // threads per row (a level with few parents: shorter dependent chains, more

@@ -2092,6 +2092,7 @@ static inline unsigned fine_wgrid(const msmg_ctx* c, int W = kWarpsPerCta) {
 //               16x2x2 143 / 47, 16x8x4 63 / 76
 //   FP32 post   4x4x5 164 / 59, 6x6x6 110 / 92, 8x8x4 94 / 65; 6x6x8 91 / 112, 7x7x7 99 / 113;
 //               lines of 5 and 7, swept out of shared memory: 5x5x5 144 / 113, 5x5x8 110 / 116
+//               (an iteration with 512 elements of 5x5x5 85 / 88, with 1000 96 / 92)
 //   FP64 pre    4x4x5 149 / 76, 6x6x6 108 / 88; 8x8x4 92 / 108, 8x8x6 99 / 167
 //   FP64 post   4x4x5 285 / 138, 4x6x6 214 / 153; 6x6x6 187 / 197, 8x8x4 167 / 266
 //   pmatvec     4x4x5 80 / 53, 6x6x6 55 / 46, 8x8x4 58 / 57; 8x8x6 49 / 50
@@ -2110,7 +2111,8 @@ static bool use_groups(const msmg_ctx* c, const G& g) {
   if (IsCube8<G>::value || g.by > 16 || (!f32 && !many)) return false;
   auto up_to = [&](int cells) { return g.nb <= (g.bx <= 8 ? cells : 96); };
   if (K == kGrpPre) return f32 ? up_to(512) && !IsGeoC<G>::value : up_to(216);
-  if (K == kGrpPost) return f32 ? up_to(g.bx == 5 || g.bx == 7 ? 128 : 256) : up_to(144) && g.bz <= 16;
+  if (K == kGrpPost && f32 && (g.bx == 5 || g.bx == 7)) return up_to(128) && c->fine.m >= 152 * 5;
+  if (K == kGrpPost) return f32 ? up_to(256) : up_to(144) && g.bz <= 16;
   if (K == kGrpPmatvec) return up_to(256) && g.by <= 12 && g.bz <= 12;
   return many && !IsGeoC<G>::value && (f32 || g.bz <= 16);   // restrict: not on 4^3, two full cells a lane
 }

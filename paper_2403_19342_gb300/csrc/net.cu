@@ -68,7 +68,8 @@ namespace msmg {
 // ------------------------------------------------------------------ CUDA-core product
 // C = epi(A[M][K] B[K][N] + bias), BF16 operands, FP32 accumulation, for the forward
 // pass of networks whose widths are not multiples of 64.  Each output is one chain of
-// fmaf over k = 0 .. K-1, whatever the tile.  256 threads, TM x TN outputs each; the next K block is in registers while this one is multiplied.
+// fmaf over k = 0 .. K-1, whatever the tile.  256 threads, TM x TN outputs each; the next K
+// block is in registers while this one is multiplied.
 //   EPI 2: ReLU, stored in BF16 (the next layer's operand); EPI 3: times wgt[m][n mod n_in], FP32.
 template <int BM, int BN, int BK, int TM, int TN, int EPI>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
